@@ -46,15 +46,9 @@ struct FFTDesc {
     int tws[WSC_MAX_STAGES];                  // L / (Ns R)
     int toff[WSC_MAX_STAGES];                 // offset of stage s's twiddle block in the table
     int tw_len;                               // complex entries of the whole table
-    int tw_full16;                            // radix-16 stages hold all fifteen powers (FP64)
     unsigned long long mag[WSC_MAX_STAGES];  // ceil(2^40 / Ns): j / Ns == (j * mag) >> 40 for j < 2^24, Ns < 2^16
 };
 
-// Compile-time lengths whose shared-memory twiddle table holds every stage's blocks but the last
-// stage's: FP64 L = 2^13, whose full table (131 KB) does not fit beside the 139 KB line; the last,
-// radix-2 stage (one power per butterfly) reads the global table.
-__host__ __device__ constexpr bool tw_split_ed(int ed, int elem_bytes) { return elem_bytes == 8 && ed == 1013; }
-template <typename T, int ED> __host__ __device__ constexpr bool tw_split_ok() { return tw_split_ed(ED, (int)sizeof(T)); }
 // Compile-time lengths whose split R2C column pass may run with one buffer per CTA: those of the
 // 512-thread kernels (at L = 2^14, 1024 threads of 64 registers, that kernel spills 600 B).
 __host__ __device__ constexpr bool split_one_ed(int ed) { return ed >= 1000 && ed != 1014; }
@@ -296,9 +290,8 @@ template <int R, bool INV, typename V> __device__ __forceinline__ void dftR(V *x
 }
 
 // ---------------------------------------------------------------- twiddles
-// x[q] *= w^{qk}, q = 1..R-1, from the stage's blocks (k < Ns): radices 2..8, and radix 16 in FP32,
-// read [w^k | w^{2k} | w^{4k} (| w^{8k})] (the blocks they need) and form the other powers as
-// products; FP64 radix 16 reads all fifteen powers [w^k | w^{2k} | ... | w^{15k}].
+// x[q] *= w^{qk}, q = 1..R-1, from the stage's blocks (k < Ns) [w^k | w^{2k} | w^{4k} (| w^{8k})] (those
+// the radix needs); the other powers are products.
 template <typename T, bool TWS>
 __device__ __forceinline__ typename cvec<T>::t tw_load(const typename cvec<T>::t *__restrict__ tw, int t)
 {
@@ -311,17 +304,6 @@ __device__ __forceinline__ void apply_twiddles(typename cvec<T>::t *x, const typ
                                                int Ns, int k)
 {
     typedef typename cvec<T>::t V;
-    if constexpr (R == 16 && sizeof(T) == 8) {
-        // FP64 radix 16 reads all fifteen powers (block q-1 holds w^{qk}): its FP64 units are the
-        // bound, and loads cost less than eleven complex products
-#pragma unroll
-        for (int q = 1; q < 16; ++q) {
-            V w = tw_load<T, TWS>(tab, (q - 1) * Ns + k);
-            if (INV) w.y = -w.y;
-            x[q] = cmul(x[q], w);
-        }
-        return;
-    }
     V w1 = tw_load<T, TWS>(tab, k);
     if (INV) w1.y = -w1.y;
     x[1] = cmul(x[1], w1);
@@ -342,7 +324,7 @@ __device__ __forceinline__ void apply_twiddles(typename cvec<T>::t *x, const typ
     x[6] = cmul(x[6], w6);
     x[7] = cmul(x[7], w7);
     if constexpr (R == 8) return;
-    // FP32 radix 16: a fourth block w^{8k}; powers 9..15 = (1..7) + 8
+    // radix 16: a fourth block w^{8k}; powers 9..15 = (1..7) + 8
     V w8 = tw_load<T, TWS>(tab, 3 * Ns + k);
     if (INV) w8.y = -w8.y;
     x[8] = cmul(x[8], w8);

@@ -29,11 +29,11 @@
 
 namespace wsc {
 
-__host__ __device__ constexpr int tw_blocks_c(int R, bool full16) { return R == 2 ? 1 : (R <= 4 ? 2 : (R <= 8 ? 3 : (full16 ? 15 : 4))); }
+__host__ __device__ constexpr int tw_blocks_c(int R) { return R == 2 ? 1 : (R <= 4 ? 2 : (R <= 8 ? 3 : 4)); }
 
 // Stage structure of compile-time length ED (the host's factorize gives the same sequence and
 // twiddle table: with radix16 set for ED = 1000 + l, with E = 24 for ED = 2000 + l).
-template <int ED, bool FULL16 = false> struct StaticStages {
+template <int ED> struct StaticStages {
     static constexpr bool X3 = ED >= 2000;                     // L = 3 2^L2
     static constexpr int L2 = X3 ? ED - 2000 : ED - 1000;      // log2 of the power-of-two factor
     static constexpr int L = X3 ? 3 << L2 : 1 << L2;
@@ -51,7 +51,7 @@ template <int ED, bool FULL16 = false> struct StaticStages {
     __host__ __device__ static constexpr int toff(int s)
     {
         int o = 0;
-        for (int i = 0; i < s; ++i) o += tw_blocks_c(R(i), FULL16) << lNs(i);
+        for (int i = 0; i < s; ++i) o += tw_blocks_c(R(i)) << lNs(i);
         return o;
     }
 };
@@ -67,7 +67,7 @@ __device__ __forceinline__ void sstage(const typename cvec<T>::t *bin, typename 
                                        const Dst &dst)
 {
     typedef typename cvec<T>::t V;
-    typedef StaticStages<ED, sizeof(T) == 8> P;  // FP64 tables hold all fifteen radix-16 powers
+    typedef StaticStages<ED> P;
     constexpr int R = P::R(S), lNs = P::lNs(S), Ns = 1 << lNs, RN = R * Ns;
     constexpr int TPT = P::L / E, NB = E / R, NBF = NB * TPT;
     constexpr int PS = pad_shift<T>::v, PAD = 1 << PS;
@@ -150,44 +150,39 @@ template <typename T, int E, int ED, bool INV, bool TWS, bool HIN, bool HOUT, bo
           int S>
 __device__ __forceinline__ void fft_static_from(typename cvec<T>::t *b0, typename cvec<T>::t *b1,
                                                 const typename cvec<T>::t *__restrict__ tw,
-                                                const typename cvec<T>::t *__restrict__ twg, int lt, const Src &src,
+                                        int lt, const Src &src,
                                                 const Dst &dst, const After0 &after0)
 {
     constexpr int NST = StaticStages<ED>::NST;
     static_assert(NST >= 2, "at least two stages");
     // stage S reads X_S and writes X_{S+1}
     typename cvec<T>::t *bin = (S & 1) ? b1 : b0, *bout = (S & 1) ? b0 : b1;
-    // a table split between shared and global memory: the last stage reads the global one
-    constexpr bool GLOBAL_TW = TWS && S == NST - 1 && tw_split_ok<T, ED>();
-    constexpr bool TWS_S = TWS && !GLOBAL_TW;
-    const typename cvec<T>::t *tws = GLOBAL_TW ? twg : tw;
     // keep each stage's per-thread bases from being hoisted to the kernel start (register pressure)
     int lt_ = lt;
     asm volatile("" : "+r"(lt_));
     if constexpr (S == 0) {
-        sstage<T, E, ED, 0, INV, TWS_S, HIN, HOUT, PP>(bin, bout, tws, lt_, src, ToSmem{});
+        sstage<T, E, ED, 0, INV, TWS, HIN, HOUT, PP>(bin, bout, tw, lt_, src, ToSmem{});
         after0();
     } else if constexpr (S == NST - 1) {
-        sstage<T, E, ED, S, INV, TWS_S, HIN, HOUT, PP>(bin, bout, tws, lt_, FromSmem{}, dst);
+        sstage<T, E, ED, S, INV, TWS, HIN, HOUT, PP>(bin, bout, tw, lt_, FromSmem{}, dst);
     } else {
-        sstage<T, E, ED, S, INV, TWS_S, HIN, HOUT, PP>(bin, bout, tws, lt_, FromSmem{}, ToSmem{});
+        sstage<T, E, ED, S, INV, TWS, HIN, HOUT, PP>(bin, bout, tw, lt_, FromSmem{}, ToSmem{});
     }
     if constexpr (S + 1 < NST)
-        fft_static_from<T, E, ED, INV, TWS, HIN, HOUT, PP, Src, Dst, After0, S + 1>(b0, b1, tw, twg, lt, src, dst,
+        fft_static_from<T, E, ED, INV, TWS, HIN, HOUT, PP, Src, Dst, After0, S + 1>(b0, b1, tw, lt, src, dst,
                                                                                    after0);
 }
 
 // Whole transform of compile-time length ED; same contract as fft_fused.  Shared-memory inputs
 // (FromSmem) are read from b0; shared-memory outputs end in X_NST (final_buf).  b1 = b0 without PP.
-// tw: the twiddle table (shared memory with TWS); twg: the global table, which the last stage
-// reads when the shared copy holds only the earlier stages' blocks (tw_split_ok).
+// tw: the twiddle table (shared memory with TWS).
 template <typename T, int E, int ED, bool INV, bool TWS, bool HIN, bool HOUT, bool PP, class Src, class Dst, class After0>
 __device__ __forceinline__ void fft_static(typename cvec<T>::t *b0, typename cvec<T>::t *b1,
                                            const typename cvec<T>::t *__restrict__ tw,
-                                           const typename cvec<T>::t *__restrict__ twg, int lt, const Src &src,
+                                        int lt, const Src &src,
                                            const Dst &dst, const After0 &after0)
 {
-    fft_static_from<T, E, ED, INV, TWS, HIN, HOUT, PP, Src, Dst, After0, 0>(b0, b1, tw, twg, lt, src, dst, after0);
+    fft_static_from<T, E, ED, INV, TWS, HIN, HOUT, PP, Src, Dst, After0, 0>(b0, b1, tw, lt, src, dst, after0);
 }
 
 // The buffer holding a compile-time transform's shared-memory outputs, X_NST, and the other one.
@@ -201,10 +196,10 @@ template <typename T, int E, int ED, bool INV, bool TWS, bool HIN = false, bool 
           class After0 = NoHook>
 __device__ __forceinline__ void fft_any(typename cvec<T>::t *buf, const FFTDesc *__restrict__ P,
                                         const typename cvec<T>::t *__restrict__ tw,
-                                        const typename cvec<T>::t *__restrict__ twg, int lt, int tpt, const Src &src,
+                                        int lt, int tpt, const Src &src,
                                         const Dst &dst, const After0 &after0 = After0{})
 {
-    if constexpr (ED >= 1000) fft_static<T, E, ED, INV, TWS, HIN, HOUT, false>(buf, buf, tw, twg, lt, src, dst, after0);
+    if constexpr (ED >= 1000) fft_static<T, E, ED, INV, TWS, HIN, HOUT, false>(buf, buf, tw, lt, src, dst, after0);
     else fft_fused<T, E, ED, INV, TWS>(buf, P, tw, lt, tpt, src, dst, after0);
 }
 
@@ -214,10 +209,10 @@ template <typename T, int E, int ED, bool INV, bool TWS, bool HIN, bool HOUT, bo
           class After0 = NoHook>
 __device__ __forceinline__ void fft_any2(typename cvec<T>::t *b0, typename cvec<T>::t *b1, const FFTDesc *__restrict__ P,
                                          const typename cvec<T>::t *__restrict__ tw,
-                                         const typename cvec<T>::t *__restrict__ twg, int lt, int tpt, const Src &src,
+                                        int lt, int tpt, const Src &src,
                                          const Dst &dst, const After0 &after0 = After0{})
 {
-    if constexpr (ED >= 1000) fft_static<T, E, ED, INV, TWS, HIN, HOUT, PP>(b0, PP ? b1 : b0, tw, twg, lt, src, dst, after0);
+    if constexpr (ED >= 1000) fft_static<T, E, ED, INV, TWS, HIN, HOUT, PP>(b0, PP ? b1 : b0, tw, lt, src, dst, after0);
     else fft_fused<T, E, ED, INV, TWS>(b0, P, tw, lt, tpt, src, dst, after0);
 }
 

@@ -32,7 +32,7 @@ namespace wsc {
 // Per-thread element counts with exact (unguarded) kernels, in order of preference.  A count E
 // admits radices dividing E; FP64 prefers radix-4 stages (E = 12 or 8), FP32 radix-8 (E = 24 or
 // 16).  E = 0 is the generic guarded path (any 2^a 3^b 5^c).
-// FP64 E = 16 exists only as the compile-time-length transforms (radix 16, 128 registers)
+// FP64 E = 16 stands for the fixed-point passes (passes_fixed.cu), where they serve the length
 static const int kElems64[] = {16, 12, 24, 8, 0};
 static const int kElems32[] = {24, 16, 0};
 
@@ -88,17 +88,14 @@ static int max_threads(conv_precision prec, int E)
     } while (0)
 
 // Twiddle powers a radix-R butterfly reads from its stage's table: w^k (R = 2); w^k, w^2k (R = 3,
-// 4; w^3k is their product); w^k, w^2k, w^4k (R = 5, 8; the other powers are products); all of
-// w^k, w^2k, w^4k, w^8k (R = 16 in FP32) or all of w^k ... w^15k (R = 16 in FP64, whose FP64 units
-// are the bound).
-static inline int tw_blocks(int R, bool full16) { return R == 2 ? 1 : (R <= 4 ? 2 : (R <= 8 ? 3 : (full16 ? 15 : 4))); }
-// power of w^k that block m holds: 2^m, or m + 1 for radix 16 with all fifteen powers
-static inline long long tw_power(int R, bool full16, int m) { return R == 16 && full16 ? m + 1 : 1LL << m; }
+// 4; w^3k is their product); w^k, w^2k, w^4k (R = 5, 8; the other powers are products); w^k, w^2k,
+// w^4k, w^8k (R = 16).  Block m holds w^(2^m k).
+static inline int tw_blocks(int R) { return R == 2 ? 1 : (R <= 4 ? 2 : (R <= 8 ? 3 : 4)); }
 
 // Radix sequence for L = 2^p 3^q 5^r whose radices divide E (E = 0: any of 8, 4, 2, 3, 5):
 // power-of-two radices first (8s when allowed, else 4s), then 3s, then 5s.  radix16: a power of
 // two as radix-16 stages and one stage for the remainder (the compile-time-length transforms).
-static bool factorize(int L, int E, FFTDesc &d, bool radix16 = false, bool full16 = false)
+static bool factorize(int L, int E, FFTDesc &d, bool radix16 = false)
 {
     int rem = L, p2 = 0, p3 = 0, p5 = 0;
     while (rem % 2 == 0) { rem /= 2; ++p2; }
@@ -135,12 +132,11 @@ static bool factorize(int L, int E, FFTDesc &d, bool radix16 = false, bool full1
         d.Ns[s] = (int)Ns;
         d.tws[s] = (int)(L / (Ns * R[s]));
         d.toff[s] = off;
-        off += tw_blocks(R[s], full16) * (int)Ns;
+        off += tw_blocks(R[s]) * (int)Ns;
         d.mag[s] = ((1ULL << 40) + (unsigned long long)Ns - 1) / (unsigned long long)Ns;
         Ns *= R[s];
     }
     d.tw_len = off;
-    d.tw_full16 = full16 ? 1 : 0;
     return true;
 }
 
@@ -152,9 +148,9 @@ void stage_twiddles(const FFTDesc &d, std::vector<double> &re_im)
     re_im.assign(2 * (size_t)d.tw_len, 0.0);
     for (int s = 0; s < d.nst; ++s) {
         const long long Ns = d.Ns[s], NR = Ns * d.R[s];
-        for (int m = 0; m < tw_blocks(d.R[s], d.tw_full16); ++m)
+        for (int m = 0; m < tw_blocks(d.R[s]); ++m)
             for (long long k = 0; k < Ns; ++k) {
-                const long long e = (tw_power(d.R[s], d.tw_full16, m) * k) % NR;
+                const long long e = ((1LL << m) * k) % NR;
                 const long double ang = 2.0L * PI_L * (long double)e / (long double)NR;
                 const size_t i = (size_t)d.toff[s] + (size_t)m * Ns + (size_t)k;
                 re_im[2 * i] = (double)cosl(ang);
@@ -188,22 +184,6 @@ static int generic_tpt(const FFTDesc &P)
         else if ((prec) == CONV_P_FP32 && (E) == 16 && (ED) == 130) { \
             if (tws) { typedef float T_; constexpr int E_ = 16, ED_ = 130; constexpr bool W_ = true; CALL; } \
             else { typedef float T_; constexpr int E_ = 16, ED_ = 130; constexpr bool W_ = false; CALL; } \
-        } \
-        else if ((prec) == CONV_P_FP64 && (E) == 16 && (ED) == 1010) { \
-            if (tws) { typedef double T_; constexpr int E_ = 16, ED_ = 1010; constexpr bool W_ = true; CALL; } \
-            else { typedef double T_; constexpr int E_ = 16, ED_ = 1010; constexpr bool W_ = false; CALL; } \
-        } \
-        else if ((prec) == CONV_P_FP64 && (E) == 16 && (ED) == 1011) { \
-            if (tws) { typedef double T_; constexpr int E_ = 16, ED_ = 1011; constexpr bool W_ = true; CALL; } \
-            else { typedef double T_; constexpr int E_ = 16, ED_ = 1011; constexpr bool W_ = false; CALL; } \
-        } \
-        else if ((prec) == CONV_P_FP64 && (E) == 16 && (ED) == 1012) { \
-            if (tws) { typedef double T_; constexpr int E_ = 16, ED_ = 1012; constexpr bool W_ = true; CALL; } \
-            else { typedef double T_; constexpr int E_ = 16, ED_ = 1012; constexpr bool W_ = false; CALL; } \
-        } \
-        else if ((prec) == CONV_P_FP64 && (E) == 16 && (ED) == 1013) { \
-            if (tws) { typedef double T_; constexpr int E_ = 16, ED_ = 1013; constexpr bool W_ = true; CALL; } \
-            else { typedef double T_; constexpr int E_ = 16, ED_ = 1013; constexpr bool W_ = false; CALL; } \
         } \
         else if ((prec) == CONV_P_FP32 && (E) == 16 && (ED) == 1008) { \
             if (tws) { typedef float T_; constexpr int E_ = 16, ED_ = 1008; constexpr bool W_ = true; CALL; } \
@@ -284,10 +264,6 @@ static int generic_tpt(const FFTDesc &P)
     } while (0)
 
 static const int kFusedSets[][3] = {
-    {0, 16, 1010},  // FP64 compile-time power-of-two lengths 2^10 ... 2^13
-    {0, 16, 1011},
-    {0, 16, 1012},
-    {0, 16, 1013},
     {1, 16, 1008},  // FP32 compile-time power-of-two lengths 2^8 ... 2^14
     {1, 16, 1009},
     {1, 16, 1010},
@@ -401,14 +377,6 @@ static int default_options(const conv_plan_s *p, int ed, int pass)
     // L = 2^14 at 1024 threads: 32 warps per SM hide the latency a prefetch would, and its staging
     // does not fit beside the 139 KB line (n = 8192, batch 8: 16.2 -> 15.4 ms per batch)
     if (ed == 1014) return 0;
-    // FP64 column passes: twiddles in shared memory.  Read through L1, the fifteen powers a
-    // radix-16 butterfly loads are hoisted into registers and the kernel spills (556 B a thread at
-    // L = 2^13), whose write-backs doubled its DRAM writes (9.2 GB against 4.3 GB algorithmic per
-    // launch at n = 4096, batch 16); from shared memory it does not spill, at +0.4 % time.  At
-    // L = 2^13 only the radix-16 stages' blocks fit beside the line (tw_split_ed), without room for
-    // the prefetch (which made no measurable difference there).
-    if (ed >= 1000 && ed < 2000 && p->prec == CONV_P_FP64 && pass == 1)
-        return tw_split_ed(ed, 8) ? CFG_TWS : CFG_TWS | CFG_PF;
     if (ed >= 1000) return pass == 2 ? (pairs ? CFG_PF | CFG_TMA : CFG_TWS) : CFG_PF;
     if (!pairs) return pass == 2 ? 0 : CFG_TWS;
     return pass == 1 ? CFG_TWS : CFG_TWS | CFG_PF | CFG_TMA;
@@ -423,6 +391,11 @@ static bool configure(conv_plan_s *p, const Candidate &c, int smem_optin, int sm
 {
     const int E = c[0], fused_pref = c[1];
     const int M = p->M, n = p->n;
+    p->fixed = false;
+    // FP64 lines of 32 to 8192 points (as far as two buffers fit beside each other, for the lengths
+    // without kernels of their own) run in fixed point: 3.6 to 4.7 times the FP64 stages' rate from n = 256 on,
+    // 1.6 times at n = 64 (n = 4096, batch 16: 125.3 -> 27.6 ms; n = 480, period 3, batch 8: 2266 -> 592 us)
+    if (p->prec == CONV_P_FP64 && E == 16) return fused_pref == 1 && fixed_configure(p, smem_optin, sms);
     const size_t esz = p->prec == CONV_P_FP64 ? 16 : 8;
     const size_t per = (size_t)(p->prec == CONV_P_FP64 ? padded_len<double>(M) : padded_len<float>(M)) * esz;
     FFTDesc d;
@@ -440,16 +413,14 @@ static bool configure(conv_plan_s *p, const Candidate &c, int smem_optin, int sm
     // extension and the crop)
     const int ed = fused_pref != 0 ? fused_edges(p->prec, E, d, fused_pref == 1 ? n : 0) : 0;
     const bool fused = ed != 0;
-    if (p->prec == CONV_P_FP64 && E == 16 && ed < 1000) return false;  // no runtime FP64 E = 16 kernels
     if (ed >= 1000) {
         // the compile-time-length kernels: radix-16 stages (L = 2^l; radix 8 and 3 for L = 3 2^l,
         // as factorize gives already), their launch bound
-        if (ed < 2000 && !factorize(M, E, d, true, p->prec == CONV_P_FP64)) return false;
+        if (ed < 2000 && !factorize(M, E, d, true)) return false;
         maxT = std::min(maxT, static_max_threads(ed));
         if (tpt > maxT) return false;
     }
-    // twiddle bytes in shared memory (TWS): the whole table, or all but the last stage's blocks
-    const size_t twb = (size_t)(tw_split_ed(ed, (int)(esz / 2)) ? d.toff[d.nst - 1] : d.tw_len) * esz;
+    const size_t twb = (size_t)d.tw_len * esz;  // the table in shared memory (TWS)
     // Staging per group (fused passes), by pass:
     //   pass 1: prefetched input rows (n elements V, rounded to 128 B), then with TMA stores the
     //           row pair's spectrum pairs, nbox x TMA_ROWS x 2 elements;
@@ -509,7 +480,7 @@ static bool configure(conv_plan_s *p, const Candidate &c, int smem_optin, int sm
     for (int k = 0; k < 3; ++k) opt[k] = c[2 + k] == CFG_DEFAULT ? default_options(p, ed, k) : c[2 + k];
     LaunchShape R, C, I;
     // R2C with complex ghat runs the split pipeline when its pass 2 fits two buffers per CTA.
-    // Where two lines do not fit one CTA (FP64 at L = 8192), the compile-time lengths run it with
+    // Where two lines do not fit one CTA, the compile-time lengths run it with
     // one buffer and a global scratch line per CTA group (after the spectra in the workspace:
     // workspace_bytes counts them).  Otherwise the C2C layout.
     const bool cplx_r2c = p->io == CONV_IO_R2C && p->complex_ghat;
@@ -580,6 +551,7 @@ static conv_status device_limits(conv_plan_s *p, int &smem_optin, int &sms)
         std::lock_guard<std::mutex> lk(mu);
         if (!attrs_set[dev]) {
             conv_status rc = set_all_attrs(smem_optin);
+            if (rc == CONV_OK) rc = set_all_attrs_fixed(smem_optin);
             if (rc != CONV_OK) return rc;
             attrs_set[dev] = true;
         }
@@ -700,6 +672,7 @@ conv_status launch_pipeline(conv_plan_s *p, const void *u, const void *mask, voi
                             double alpha_re, double alpha_im, double beta, void *ws, cudaStream_t st)
 {
     if (p->long_lines) return long_lines_apply(p, u, mask, out, batch, alpha_re, alpha_im, beta, ws, st);
+    if (p->fixed) return launch_fixed(p, u, mask, out, batch, alpha_re, alpha_im, beta, ws, st);
     conv_status rc = CONV_OK;
     if (p->fused)
         WSC_DISPATCH_FUSED(p->prec, p->elems, p->ed, false,

@@ -156,7 +156,7 @@ __global__ void WSC_LBF(T, E, ED) kf_r2r_rows_fwd(const __grid_constant__ PassAr
             }
             return cmk<V>(x, y);
         };
-        fft_any2<T, E, ED, false, TWS, pruned<ED>(), false, PP>(buf, buf2, a.P, twp, a.tw, lt, a.tpt, src, ToSmem{},
+        fft_any2<T, E, ED, false, TWS, pruned<ED>(), false, PP>(buf, buf2, a.P, twp, lt, a.tpt, src, ToSmem{},
                                                                 [&]() { fetch(unit + stride); });
         const V *spec = (PP && final_in_b1<ED>()) ? buf2 : buf;  // the spectrum Z
         if (a.tma) {
@@ -240,16 +240,16 @@ __global__ void WSC_LBF(T, E, ED) kf_r2r_cols(const __grid_constant__ PassArgs<T
             const int Lm = pruned<ED>() ? static_len<ED>() : M, k1 = o <= Lm / 2 ? o : Lm - o;
             x = a.odd ? odd_mul(x, __ldg(&gc[k1]), o, Lm) : cscale(x, __ldg(&gc[k1]));
         });
-        fft_any2<T, E, ED, false, TWS, pruned<ED>(), false, PP>(buf, buf2, a.P, twp, a.tw, lt, a.tpt, src, mul,
+        fft_any2<T, E, ED, false, TWS, pruned<ED>(), false, PP>(buf, buf2, a.P, twp, lt, a.tpt, src, mul,
                                                                 [&]() { fetch(unit + stride); });
         auto dst = [&](int o, V x) {
             if (valid && o < n) col[o] = x;
         };
         // the inverse starts from the buffer the forward transform ended in
         if (final_in_b1<ED>() && PP)
-            fft_any2<T, E, ED, true, TWS, false, pruned<ED>(), PP>(buf2, buf, a.P, twp, a.tw, lt, a.tpt, FromSmem{}, dst);
+            fft_any2<T, E, ED, true, TWS, false, pruned<ED>(), PP>(buf2, buf, a.P, twp, lt, a.tpt, FromSmem{}, dst);
         else
-            fft_any2<T, E, ED, true, TWS, false, pruned<ED>(), PP>(buf, buf2, a.P, twp, a.tw, lt, a.tpt, FromSmem{}, dst);
+            fft_any2<T, E, ED, true, TWS, false, pruned<ED>(), PP>(buf, buf2, a.P, twp, lt, a.tpt, FromSmem{}, dst);
         __syncthreads();
     }
 }
@@ -344,7 +344,7 @@ __global__ void WSC_LBF(T, E, ED) kf_r2r_rows_inv(const __grid_constant__ PassAr
             oa[o] = ra;
             if (has2) oa[n + o] = rb;
         };
-        fft_any2<T, E, ED, true, TWS, false, pruned<ED>(), PP>(buf, buf2, a.P, twp, a.tw, lt, a.tpt, src, dst,
+        fft_any2<T, E, ED, true, TWS, false, pruned<ED>(), PP>(buf, buf2, a.P, twp, lt, a.tpt, src, dst,
                                                                [&]() { gather(unit + stride); });
         __syncthreads();
     }
@@ -369,7 +369,7 @@ __global__ void WSC_LBF(T, E, ED) kf_r2c_cols(const __grid_constant__ PassArgs<T
     typedef typename cvec<T>::t V;
     const int g = threadIdx.x / a.tpt, lt = threadIdx.x - g * a.tpt, G = blockDim.x / a.tpt;
     const V *twp;
-    // ONE: a single buffer per group (two lines do not fit, FP64 at L = 8192); the Im-ghat
+    // ONE: a single buffer per group (the lines that leave no room for two); the Im-ghat
     // spectrum waits in the group's global scratch line, in L2, while the Re part is inverted
     V *bre = setup_smem<T, TWS>(a, twp, ONE ? g : 2 * g);
     V *bim = ONE ? nullptr : bre + padded_len<T>(a.M);
@@ -411,7 +411,7 @@ __global__ void WSC_LBF(T, E, ED) kf_r2c_cols(const __grid_constant__ PassArgs<T
             else bim[pidx<T>(o)] = cscale(x, gk.y);
             x = cscale(x, gk.x);
         });
-        fft_any<T, E, ED, false, TWS, pruned<ED>(), false>(bre, a.P, twp, a.tw, lt, a.tpt, src, mul, [&]() { fetch(unit + stride); });
+        fft_any<T, E, ED, false, TWS, pruned<ED>(), false>(bre, a.P, twp, lt, a.tpt, src, mul, [&]() { fetch(unit + stride); });
         V *cout = reinterpret_cast<V *>(a.out) + 2 * co;
         if constexpr (ONE) {
             // Wr straight to the output pairs' first halves; then Wi from the scratch line (its
@@ -419,17 +419,17 @@ __global__ void WSC_LBF(T, E, ED) kf_r2c_cols(const __grid_constant__ PassArgs<T
             auto dst_r = [&](int o, V xr) {
                 if (valid && o < n) cout[2 * o] = xr;
             };
-            fft_any<T, E, ED, true, TWS, false, pruned<ED>()>(bre, a.P, twp, a.tw, lt, a.tpt, FromSmem{}, dst_r);
+            fft_any<T, E, ED, true, TWS, false, pruned<ED>()>(bre, a.P, twp, lt, a.tpt, FromSmem{}, dst_r);
             __syncthreads();
             auto src_i = [&](int i) -> V { return tmp[i]; };
             auto dst_i = [&](int o, V xi) {
                 if (valid && o < n) cout[2 * o + 1] = xi;
             };
-            fft_any<T, E, ED, true, TWS, false, pruned<ED>()>(bre, a.P, twp, a.tw, lt, a.tpt, src_i, dst_i);
+            fft_any<T, E, ED, true, TWS, false, pruned<ED>()>(bre, a.P, twp, lt, a.tpt, src_i, dst_i);
             __syncthreads();
             continue;
         }
-        fft_any<T, E, ED, true, TWS, false, pruned<ED>()>(bre, a.P, twp, a.tw, lt, a.tpt, FromSmem{}, ToSmem{});
+        fft_any<T, E, ED, true, TWS, false, pruned<ED>()>(bre, a.P, twp, lt, a.tpt, FromSmem{}, ToSmem{});
         auto dst = [&](int o, V xi) {
             if (!valid || o >= n) return;
             const V xr = bre[pidx<T>(o)];
@@ -442,7 +442,7 @@ __global__ void WSC_LBF(T, E, ED) kf_r2c_cols(const __grid_constant__ PassArgs<T
             cout[2 * o] = xr;
             cout[2 * o + 1] = xi;
         };
-        fft_any<T, E, ED, true, TWS, false, pruned<ED>()>(bim, a.P, twp, a.tw, lt, a.tpt, FromSmem{}, dst);
+        fft_any<T, E, ED, true, TWS, false, pruned<ED>()>(bim, a.P, twp, lt, a.tpt, FromSmem{}, dst);
         __syncthreads();
     }
 }
@@ -522,7 +522,7 @@ __global__ void WSC_LBF(T, E, ED) kf_r2c_rows_inv(const __grid_constant__ PassAr
             if (a.beta != (T)0) z.x += a.beta * ua[o];
             o_[o] = z;
         };
-        fft_any<T, E, ED, true, TWS, false, pruned<ED>()>(buf, a.P, twp, a.tw, lt, a.tpt, src, dst, [&]() { gather(unit + stride); });
+        fft_any<T, E, ED, true, TWS, false, pruned<ED>()>(buf, a.P, twp, lt, a.tpt, src, dst, [&]() { gather(unit + stride); });
         __syncthreads();
     }
     if (a.pf) cp_async_wait_all();
@@ -573,7 +573,7 @@ __global__ void WSC_LBF(T, E, ED) kf_c2c_rows_fwd(const __grid_constant__ PassAr
         auto dst = [&](int o, V z) {
             if (valid) Wb[(size_t)o * n + j1] = z;
         };
-        fft_any<T, E, ED, false, TWS, pruned<ED>(), false>(buf, a.P, twp, a.tw, lt, a.tpt, src, dst, [&]() { fetch(unit + stride); });
+        fft_any<T, E, ED, false, TWS, pruned<ED>(), false>(buf, a.P, twp, lt, a.tpt, src, dst, [&]() { fetch(unit + stride); });
         __syncthreads();
     }
 }
@@ -620,11 +620,11 @@ __global__ void WSC_LBF(T, E, ED) kf_c2c_cols(const __grid_constant__ PassArgs<T
             if (CG) x = cmul(x, __ldg(reinterpret_cast<const V *>(gq) + (size_t)k2q * h + k1));
             else x = cscale(x, __ldg(reinterpret_cast<const T *>(gq) + (size_t)k2q * h + k1));
         });
-        fft_any<T, E, ED, false, TWS, pruned<ED>(), false>(buf, a.P, twp, a.tw, lt, a.tpt, src, mul, [&]() { fetch(unit + stride); });
+        fft_any<T, E, ED, false, TWS, pruned<ED>(), false>(buf, a.P, twp, lt, a.tpt, src, mul, [&]() { fetch(unit + stride); });
         auto dst = [&](int o, V x) {
             if (valid && o < n) col[o] = x;
         };
-        fft_any<T, E, ED, true, TWS, false, pruned<ED>()>(buf, a.P, twp, a.tw, lt, a.tpt, FromSmem{}, dst);
+        fft_any<T, E, ED, true, TWS, false, pruned<ED>()>(buf, a.P, twp, lt, a.tpt, FromSmem{}, dst);
         __syncthreads();
     }
 }
@@ -676,7 +676,7 @@ __global__ void WSC_LBF(T, E, ED) kf_c2c_rows_inv(const __grid_constant__ PassAr
             }
             o_[o] = z;
         };
-        fft_any<T, E, ED, true, TWS, false, pruned<ED>()>(buf, a.P, twp, a.tw, lt, a.tpt, src, dst, [&]() { gather(unit + stride); });
+        fft_any<T, E, ED, true, TWS, false, pruned<ED>()>(buf, a.P, twp, lt, a.tpt, src, dst, [&]() { gather(unit + stride); });
         __syncthreads();
     }
     if (a.pf) cp_async_wait_all();
@@ -735,7 +735,7 @@ conv_status run_fused(conv_plan_s *p, const void *u, const void *mask, void *out
     a.ghat = p->prec == CONV_P_FP64 ? (const void *)p->ghat64 : p->ghat32;
     a.u = u;
     a.tw = reinterpret_cast<const V *>(p->tw);
-    a.tw_len = tw_split_ok<T, ED>() ? p->fft.toff[p->fft.nst - 1] : p->fft.tw_len;  // the shared-memory copy
+    a.tw_len = p->fft.tw_len;
     a.P = p->fft_dev;
     a.n = n;
     a.h = h;

@@ -83,6 +83,17 @@ void stage_twiddles(const FFTDesc &d, std::vector<double> &re_im);
 static conv_status upload_twiddles(conv_plan_s *p)
 {
     if (p->long_lines) return CONV_OK;  // the long-line pipeline keeps its own tables
+    if (p->fixed) {
+        std::vector<int> t;
+        fixed_twiddles(p->fixed_desc, t);
+        if (dev_alloc(&p->tw, t.size() * sizeof(int)) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(CONV_ENOMEM, "cudaMalloc of the twiddle table failed");
+        }
+        WSC_CUDA(cudaMemcpyAsync(p->tw, t.data(), t.size() * sizeof(int), cudaMemcpyHostToDevice, p->setup_stream));
+        WSC_CUDA(cudaStreamSynchronize(p->setup_stream));
+        return CONV_OK;
+    }
     std::vector<double> h;
     stage_twiddles(p->fft, h);
     const bool f64 = p->prec == CONV_P_FP64;

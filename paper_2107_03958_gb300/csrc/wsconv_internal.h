@@ -74,6 +74,21 @@ enum { CFG_TWS = 1, CFG_PF = 2, CFG_ONE = 4, CFG_TMA = 8, CFG_DEFAULT = -1 };
 // tma.cu
 bool encode_rows_map(CUtensorMap *m, const void *base, unsigned long long words, unsigned long long rows,
                      unsigned long long batch, unsigned box_words);
+#define FIXED_MAX_STAGES 12
+
+// Stage structure of one fixed-point transform (kernel parameter).  The first stage has no
+// twiddles; the powers of two come first (16s, then the rest), so only radix-3 and radix-5 stages
+// see an Ns that is not a power of two.  Twiddle table: for stage s >= 1, tw_variants(R) copies of
+// [w^k | w^2k | ... | w^(R-1)k], k < Ns, w = exp(-2 pi i / (Ns R)), copy v scaled by 2^(62 - v): the
+// product's high word is then the product over 2^(2 + v).
+struct FixedDesc {
+    int L, nst, tw_len;
+    int R[FIXED_MAX_STAGES], Ns[FIXED_MAX_STAGES], toff[FIXED_MAX_STAGES];
+    int lg[FIXED_MAX_STAGES];                  // ceil log2 of R_1 ... R_s (growth after the first stage)
+    unsigned long long mag[FIXED_MAX_STAGES];  // ceil(2^40 / Ns)
+};
+__host__ __device__ constexpr int fixed_variants(int R) { return R == 16 ? 3 : (R == 8 || R == 5 ? 2 : 1); }
+
 // A launch configuration: {E, fused passes, options of pass 1, of pass 2, of pass 3}.  Unfused
 // passes share pass 1's twiddle option.
 typedef std::array<int, 5> Candidate;
@@ -114,6 +129,9 @@ struct conv_plan_s {
     int elems;  // complex elements per thread in the transform kernels
     bool tws;   // twiddle table staged in shared memory
     bool fused; // passes on the fused transform (global-memory first/last stages)
+    bool fixed = false;                      // FP64 passes in 64-bit fixed point (passes_fixed.cuh)
+    wsc::FixedDesc fixed_desc{};
+    int fixed_sms = 0;                       // SMs the fixed-point passes are spread over
     bool long_lines = false;                 // lines beyond one CTA: four-step FP64 pipeline (fsmask.cu)
     wsc::LongLines *longl = nullptr;
     // conv_apply_kernels: for the duration of one launch, each density's multiplier table
@@ -164,6 +182,12 @@ conv_status launch_pipeline(conv_plan_s *p, const void *u, const void *mask, voi
                             double alpha_re, double alpha_im, double beta, void *ws,
                             cudaStream_t st);
 conv_status select_transform(conv_plan_s *p);
+// passes_fixed.cu
+bool fixed_configure(conv_plan_s *p, int smem_optin, int sms);
+conv_status set_all_attrs_fixed(int smem);
+conv_status launch_fixed(conv_plan_s *p, const void *u, const void *mask, void *out, int batch, double are,
+                         double aim, double beta, void *ws, cudaStream_t st);
+void fixed_twiddles(const FixedDesc &d, std::vector<int> &tab);
 // ghat.cu
 conv_status build_ghat(conv_plan_s *p);
 conv_status copy_ghat(conv_plan_s *p, const conv_plan_s *src);  // src's FP64 tables, no recomputation
