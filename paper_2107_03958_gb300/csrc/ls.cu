@@ -19,81 +19,181 @@
 
 namespace wsc {
 
-#define LS_RED_BLOCKS 296  // 2 x 148..152 SMs: fixed partition for deterministic reductions
+#define LS_RED_BLOCKS 152  // one block per SM: fixed partition for deterministic reductions
 #define LS_RED_THREADS 256
 #define LS_MAX_RESTART 1000  // Krylov basis (restart + 1) n^2 complex values; Hessenberg (restart + 1) restart
 
-// Dot products of NV basis vectors V_i0 ... V_i0+NV-1 with w over this block's slice [lo, hi):
-// one sweep that reads w once for the NV of them.  Each thread issues the loads of four elements
-// (and of every vector) before it uses them, so enough reads are in flight to keep HBM busy;
-// the sums still run over t in the order of a plain loop, so the result is the same bit for bit.
-template <int NV>
+// The FP64 units (two lanes per SM and clock) bound these kernels: a complex multiply-add is written as
+// its four FMAs (a product sum added to the accumulator costs six instructions), and a warp's sums
+// are reduced by halving, each step adding only the values a lane keeps (a shuffle tree per value
+// costs five additions by the whole warp for each: at n = 512 three times the products themselves).
+__device__ __forceinline__ double2 as_d2(double2 v) { return v; }
+__device__ __forceinline__ double2 as_d2(float2 v) { return make_double2((double)v.x, (double)v.y); }
+// s += conj(a) b
+__device__ __forceinline__ void dot_acc(double &sr, double &si, double2 a, double2 b)
+{
+    sr = fma(a.x, b.x, sr);
+    si = fma(a.x, b.y, si);
+    sr = fma(a.y, b.y, sr);
+    si = fma(-a.y, b.x, si);
+}
+// acc + s v c
+template <int SIGN> __device__ __forceinline__ double2 axpy_acc(double2 acc, double2 v, double2 c)
+{
+    acc.x = fma(SIGN * v.x, c.x, acc.x);
+    acc.y = fma(SIGN * v.x, c.y, acc.y);
+    acc.x = fma(-SIGN * v.y, c.y, acc.x);
+    acc.y = fma(SIGN * v.y, c.x, acc.y);
+    return acc;
+}
+
+// Sums over the warp of M values per lane (M a power of two): afterwards lane l holds, in v[0], the total of
+// value l / (32 / M).
+template <int M, int OFF = 16> __device__ __forceinline__ void warp_sums(double *v, int lane)
+{
+    if constexpr (OFF > 0) {
+        if constexpr (M > 1) {
+            const bool up = (lane & OFF) != 0;
+#pragma unroll
+            for (int i = 0; i < M / 2; ++i) {
+                const double send = up ? v[i] : v[i + M / 2], keep = up ? v[i + M / 2] : v[i];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, OFF);
+            }
+            warp_sums<M / 2, OFF / 2>(v, lane);
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], OFF);
+            warp_sums<1, OFF / 2>(v, lane);
+        }
+    }
+}
+
+// Dot products of NV basis vectors V_i0 ... V_i0+NV-1 with w over this block's slice [lo, hi): one
+// sweep that reads w once for the NV of them, the loads of two elements (and of every vector) issued
+// before their use.
+template <int NV, class WT>
 __device__ __forceinline__ void dots_sweep(const double2 *__restrict__ V, size_t ldv, int i0,
-                                           const double2 *__restrict__ w, long long lo, long long hi,
-                                           double2 (*red)[LS_RED_THREADS / 32], double2 *__restrict__ partial)
+                                           const WT *__restrict__ w, long long lo, long long hi,
+                                           double (*red)[16], double2 *__restrict__ partial)
 {
     const long long S = blockDim.x;
-    double sr[NV], si[NV];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double s[2 * NV];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) sr[k] = si[k] = 0.0;
+    for (int k = 0; k < 2 * NV; ++k) s[k] = 0.0;
     long long t = lo + threadIdx.x;
-    for (; t + 3 * S < hi; t += 4 * S) {
-        double2 b[4], a[NV][4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) b[u] = w[t + u * S];
-#pragma unroll
-        for (int k = 0; k < NV; ++k)
-#pragma unroll
-            for (int u = 0; u < 4; ++u) a[k][u] = V[(size_t)(i0 + k) * ldv + t + u * S];
-#pragma unroll
-        for (int k = 0; k < NV; ++k)
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                sr[k] += a[k][u].x * b[u].x + a[k][u].y * b[u].y;
-                si[k] += a[k][u].x * b[u].y - a[k][u].y * b[u].x;
-            }
-    }
-    for (; t < hi; t += S) {
-        const double2 b = w[t];
+    for (; t + S < hi; t += 2 * S) {
+        const double2 b0 = as_d2(w[t]), b1 = as_d2(w[t + S]);
+        double2 a0[NV], a1[NV];
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
-            const double2 a = V[(size_t)(i0 + k) * ldv + t];
-            sr[k] += a.x * b.x + a.y * b.y;
-            si[k] += a.x * b.y - a.y * b.x;
+            a0[k] = V[(size_t)(i0 + k) * ldv + t];
+            a1[k] = V[(size_t)(i0 + k) * ldv + t + S];
         }
-    }
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        for (int o = 16; o > 0; o >>= 1) {
-            sr[k] += __shfl_down_sync(0xffffffffu, sr[k], o);
-            si[k] += __shfl_down_sync(0xffffffffu, si[k], o);
+        for (int k = 0; k < NV; ++k) {
+            dot_acc(s[2 * k], s[2 * k + 1], a0[k], b0);
+            dot_acc(s[2 * k], s[2 * k + 1], a1[k], b1);
         }
-        if ((threadIdx.x & 31) == 0) red[k][threadIdx.x >> 5] = make_double2(sr[k], si[k]);
     }
+    if (t < hi) {
+        const double2 b = as_d2(w[t]);
+        double2 a[NV];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) a[k] = V[(size_t)(i0 + k) * ldv + t];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) dot_acc(s[2 * k], s[2 * k + 1], a[k], b);
+    }
+    warp_sums<2 * NV>(s, lane);
+    if ((lane & (16 / NV - 1)) == 0) red[warp][lane / (16 / NV)] = s[0];
     __syncthreads();
-    if (threadIdx.x < NV) {
-        const int k = threadIdx.x;
-        double ar = 0, ai = 0;
-        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) {
-            ar += red[k][q].x;
-            ai += red[k][q].y;
-        }
-        partial[(size_t)(i0 + k) * gridDim.x + blockIdx.x] = make_double2(ar, ai);
+    if (threadIdx.x < 2 * NV) {
+        double acc = 0;
+#pragma unroll
+        for (int q = 0; q < LS_RED_THREADS / 32; ++q) acc += red[q][threadIdx.x];
+        reinterpret_cast<double *>(partial)[2 * ((size_t)(i0 + threadIdx.x / 2) * gridDim.x + blockIdx.x) + (threadIdx.x & 1)] = acc;
     }
     __syncthreads();
 }
 
-// partial[i * nb + blk] = sum_{t in blk's slice} conj(V_i[t]) w[t], i < cnt; two vectors per sweep
+// partial[i * nb + blk] = sum_{t in blk's slice} conj(V_i[t]) w[t], i < cnt; up to eight vectors per sweep
+template <class WT>
+__device__ __forceinline__ void multidot_slice(const double2 *__restrict__ V, size_t ldv, int cnt,
+                                               const WT *__restrict__ w, long long N, double2 *__restrict__ partial)
+{
+    __shared__ double red[LS_RED_THREADS / 32][16];
+    const long long chunk = (N + gridDim.x - 1) / gridDim.x;
+    const long long lo = blockIdx.x * chunk, hi = min(N, lo + chunk);
+    int i = 0;
+    for (; i + 8 <= cnt; i += 8) dots_sweep<8>(V, ldv, i, w, lo, hi, red, partial);
+    if (cnt - i >= 4) { dots_sweep<4>(V, ldv, i, w, lo, hi, red, partial); i += 4; }
+    if (cnt - i >= 2) { dots_sweep<2>(V, ldv, i, w, lo, hi, red, partial); i += 2; }
+    if (cnt - i >= 1) dots_sweep<1>(V, ldv, i, w, lo, hi, red, partial);
+}
+
 __global__ void __launch_bounds__(LS_RED_THREADS) k_multidot(const double2 *__restrict__ V, size_t ldv, int cnt,
                                                              const double2 *__restrict__ w, long long N,
                                                              double2 *__restrict__ partial)
 {
-    __shared__ double2 red[2][LS_RED_THREADS / 32];
-    const long long chunk = (N + gridDim.x - 1) / gridDim.x;
-    const long long lo = blockIdx.x * chunk, hi = min(N, lo + chunk);
-    int i = 0;
-    for (; i + 2 <= cnt; i += 2) dots_sweep<2>(V, ldv, i, w, lo, hi, red, partial);
-    if (i < cnt) dots_sweep<1>(V, ldv, i, w, lo, hi, red, partial);
+    multidot_slice(V, ldv, cnt, w, N, partial);
+}
+
+// Whether this block is the last of the grid to arrive (every thread of it gets the answer); what the
+// others wrote before is visible to it.  The ticket is 0 before and after.
+__device__ __forceinline__ bool last_block(unsigned *ticket)
+{
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
+// Sum over the blocks of partial[i * nb + ...], nb <= 2 LS_RED_BLOCKS, by one warp; lane 0 gets it.  The loads
+// come before the sums: one by one they would cost a trip to L2 each.
+__device__ __forceinline__ double2 warp_total(const double2 *partial, int nb, int i)
+{
+    constexpr int NL = (2 * LS_RED_BLOCKS + 31) / 32;
+    const int lane = threadIdx.x & 31;
+    double2 p[NL];
+#pragma unroll
+    for (int u = 0; u < NL; ++u) {
+        const int b = lane + 32 * u;
+        p[u] = b < nb ? __ldcg(&partial[(size_t)i * nb + b]) : make_double2(0, 0);
+    }
+    double s[2] = {0, 0};
+#pragma unroll
+    for (int u = 0; u < NL; ++u)
+        if (32 * u < nb) {
+            s[0] += p[u].x;
+            s[1] += p[u].y;
+        }
+    for (int o = 16; o > 0; o >>= 1) {
+        s[0] += __shfl_down_sync(0xffffffffu, s[0], o);
+        s[1] += __shfl_down_sync(0xffffffffu, s[1], o);
+    }
+    return make_double2(s[0], s[1]);
+}
+
+// A Gram-Schmidt pass's coefficients y = V^H w, added to hcol (accumulate) or stored there: the dot
+// products, finished by the grid's last block (a step is a chain of short kernels, and two more
+// launches for the sums cost more than the sums).
+template <class WT>
+__global__ void __launch_bounds__(LS_RED_THREADS) k_gs_dots(const double2 *__restrict__ V, size_t ldv, int cnt,
+                                                            const WT *__restrict__ w, long long N, double2 *partial,
+                                                            double2 *__restrict__ hcol, int accumulate,
+                                                            double2 *__restrict__ y, unsigned *ticket)
+{
+    multidot_slice(V, ldv, cnt, w, N, partial);
+    if (!last_block(ticket)) return;
+    for (int i = threadIdx.x >> 5; i < cnt; i += LS_RED_THREADS / 32) {
+        const double2 t = warp_total(partial, gridDim.x, i);
+        if ((threadIdx.x & 31) == 0) {
+            y[i] = t;
+            hcol[i] = accumulate ? make_double2(hcol[i].x + t.x, hcol[i].y + t.y) : t;
+        }
+    }
 }
 
 // out[i] = sum_blk partial[i * nb + blk] (+= if accumulate); one warp per i, fixed order.
@@ -119,35 +219,37 @@ __global__ void k_finalize_dots(const double2 *__restrict__ partial, int nb, int
     }
 }
 
-// w -= sum_{i<cnt} V_i h_i
-__global__ void k_sub_combination(const double2 *__restrict__ V, size_t ldv, int cnt,
-                                  const double2 *__restrict__ h, double2 *__restrict__ w, long long N)
+// w = in - sum_{i<cnt} V_i h_i at element t
+template <class WT>
+__device__ __forceinline__ double2 sub_at(const double2 *__restrict__ V, size_t ldv, int cnt, const double2 *hs,
+                                          const WT *__restrict__ in, long long t)
+{
+    double2 acc = as_d2(in[t]);
+    int i = 0;
+    // four vectors' loads issued before their uses (same subtraction order as one at a time)
+    for (; i + 4 <= cnt; i += 4) {
+        double2 v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = V[(size_t)(i + k) * ldv + t];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            acc = axpy_acc<-1>(acc, v[k], hs[i + k]);
+        }
+    }
+    for (; i < cnt; ++i) acc = axpy_acc<-1>(acc, V[(size_t)i * ldv + t], hs[i]);
+    return acc;
+}
+
+// w = in - sum_{i<cnt} V_i h_i (in may be w)
+template <class WT>
+__global__ void k_sub_combination(const double2 *__restrict__ V, size_t ldv, int cnt, const double2 *__restrict__ h,
+                                  const WT *in, double2 *w, long long N)
 {
     extern __shared__ double2 hs[];  // cnt coefficients
     for (int i = threadIdx.x; i < cnt; i += blockDim.x) hs[i] = h[i];
     __syncthreads();
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < N; t += (long long)gridDim.x * blockDim.x) {
-        double2 acc = w[t];
-        int i = 0;
-        // four vectors' loads issued before their uses (same subtraction order as one at a time)
-        for (; i + 4 <= cnt; i += 4) {
-            double2 v[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) v[k] = V[(size_t)(i + k) * ldv + t];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const double2 c = hs[i + k];
-                acc.x -= v[k].x * c.x - v[k].y * c.y;
-                acc.y -= v[k].x * c.y + v[k].y * c.x;
-            }
-        }
-        for (; i < cnt; ++i) {
-            double2 v = V[(size_t)i * ldv + t], c = hs[i];
-            acc.x -= v.x * c.x - v.y * c.y;
-            acc.y -= v.x * c.y + v.y * c.x;
-        }
-        w[t] = acc;
-    }
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < N; t += (long long)gridDim.x * blockDim.x)
+        w[t] = sub_at(V, ldv, cnt, hs, in, t);
 }
 
 // x += sum_{i<cnt} V_i y_i
@@ -165,30 +267,25 @@ __global__ void k_add_combination(const double2 *__restrict__ V, size_t ldv, int
 #pragma unroll
             for (int k = 0; k < 4; ++k) v[k] = V[(size_t)(i + k) * ldv + t];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const double2 c = ys[i + k];
-                acc.x += v[k].x * c.x - v[k].y * c.y;
-                acc.y += v[k].x * c.y + v[k].y * c.x;
-            }
+            for (int k = 0; k < 4; ++k) acc = axpy_acc<1>(acc, v[k], ys[i + k]);
         }
-        for (; i < cnt; ++i) {
-            double2 v = V[(size_t)i * ldv + t], c = ys[i];
-            acc.x += v.x * c.x - v.y * c.y;
-            acc.y += v.x * c.y + v.y * c.x;
-        }
+        for (; i < cnt; ++i) acc = axpy_acc<1>(acc, V[(size_t)i * ldv + t], ys[i]);
         x[t] = acc;
     }
 }
 
-// dst = src * (1/sqrt(nrm2->x)) where nrm2 holds a squared norm (x component)
+// dst = src * nrm2->y, the inverse of the norm whose square is nrm2->x (taken once where the norm is
+// finished: a square root and a division by every thread were four fifths of this kernel's time);
+// dst32: NULL, or dst in single precision (the next FP32 matvec's input)
 __global__ void k_scale_by_invnorm(const double2 *__restrict__ src, double2 *__restrict__ dst,
-                                   const double2 *__restrict__ nrm2, long long N)
+                                   const double2 *__restrict__ nrm2, long long N, float2 *__restrict__ dst32)
 {
-    double nn = sqrt(nrm2->x);
-    double s = nn > 0 ? 1.0 / nn : 0.0;
+    const double s = nrm2->y;
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < N; t += (long long)gridDim.x * blockDim.x) {
         double2 v = src[t];
-        dst[t] = make_double2(v.x * s, v.y * s);
+        v = make_double2(v.x * s, v.y * s);
+        dst[t] = v;
+        if (dst32) dst32[t] = make_float2((float)v.x, (float)v.y);
     }
 }
 
@@ -239,8 +336,9 @@ struct GmresState {
     double2 *e;     // R + 1
     double2 *y;     // R
     double2 *hcol;  // R + 1: h of the current column (CGS accumulations)
-    double2 *nrm2;  // squared norm scratch (x component)
+    double2 *nrm2;  // a squared norm, and the norm's inverse
     double *res;    // |e[j+1]|
+    unsigned *ticket;  // blocks arrived (last_block), 0 between kernels
     int R;
 };
 
@@ -258,6 +356,7 @@ static GmresState gmres_state_view(double2 *base, int R)
     g.hcol = g.y + R;
     g.nrm2 = g.hcol + (R + 1);
     g.res = reinterpret_cast<double *>(g.nrm2 + 1);
+    g.ticket = reinterpret_cast<unsigned *>(g.res + 1);
     return g;
 }
 
@@ -266,57 +365,109 @@ __global__ void k_gmres_init(GmresState st)
 {
     if (threadIdx.x == 0) {
         for (int i = 0; i <= st.R; ++i) st.e[i] = make_double2(0, 0);
-        st.e[0] = make_double2(sqrt(st.nrm2->x), 0);
-        *st.res = sqrt(st.nrm2->x);
+        const double nn = sqrt(st.nrm2->x);
+        st.e[0] = make_double2(nn, 0);
+        *st.res = nn;
+        st.nrm2->y = nn > 0 ? 1.0 / nn : 0.0;
     }
 }
 
-// Column j of H from hcol (j+1 entries) and the new norm; apply the previous rotations, form
-// rotation j, update e and the residual estimate.
-__global__ void k_gmres_givens(GmresState st, int j, int ldh)
+// Column j of H from hcol (j+1 entries) and the new squared norm; apply the previous rotations, form
+// rotation j, update e and the residual estimate.  One block; buf: 3 (j + 1) shared elements, where the
+// column and the rotations wait for the recurrence (a chain of global loads per rotation otherwise).
+__device__ void givens_step(const GmresState &st, int j, int ldh, double nrm2, double2 *buf)
 {
-    if (threadIdx.x != 0) return;
-    for (int i = 0; i <= j; ++i) st.H[i * ldh + j] = st.hcol[i];
-    double hn = sqrt(st.nrm2->x);
-    st.H[(j + 1) * ldh + j] = make_double2(hn, 0);
-    for (int i = 0; i < j; ++i) {
-        double2 h0 = st.H[i * ldh + j], h1 = st.H[(i + 1) * ldh + j], c = st.cs[i], s = st.sn[i];
-        // [h0; h1] <- [conj(c) h0 + conj(s) h1; -s h0 + c h1]
-        double2 a = make_double2(c.x * h0.x + c.y * h0.y + s.x * h1.x + s.y * h1.y,
-                                 c.x * h0.y - c.y * h0.x + s.x * h1.y - s.y * h1.x);
-        double2 b = make_double2(-(s.x * h0.x - s.y * h0.y) + (c.x * h1.x - c.y * h1.y),
-                                 -(s.x * h0.y + s.y * h0.x) + (c.x * h1.y + c.y * h1.x));
-        st.H[i * ldh + j] = a;
-        st.H[(i + 1) * ldh + j] = b;
+    double2 *h = buf, *cs = buf + (j + 1), *sn = buf + 2 * (j + 1);
+    for (int i = threadIdx.x; i <= j; i += blockDim.x) {
+        h[i] = st.hcol[i];
+        if (i < j) {
+            cs[i] = st.cs[i];
+            sn[i] = st.sn[i];
+        }
     }
-    double2 h0 = st.H[j * ldh + j], h1 = st.H[(j + 1) * ldh + j];
-    double r = sqrt(h0.x * h0.x + h0.y * h0.y + h1.x * h1.x + h1.y * h1.y);
-    double2 c = r > 0 ? make_double2(h0.x / r, h0.y / r) : make_double2(1, 0);
-    double2 s = r > 0 ? make_double2(h1.x / r, h1.y / r) : make_double2(0, 0);
-    st.cs[j] = c;
-    st.sn[j] = s;
-    st.H[j * ldh + j] = make_double2(r, 0);
-    st.H[(j + 1) * ldh + j] = make_double2(0, 0);
-    double2 ej = st.e[j];
-    st.e[j + 1] = make_double2(-(s.x * ej.x - s.y * ej.y), -(s.x * ej.y + s.y * ej.x));
-    st.e[j] = make_double2(c.x * ej.x + c.y * ej.y, c.x * ej.y - c.y * ej.x);
-    *st.res = sqrt(st.e[j + 1].x * st.e[j + 1].x + st.e[j + 1].y * st.e[j + 1].y);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const double hn = sqrt(nrm2);
+        *st.nrm2 = make_double2(nrm2, hn > 0 ? 1.0 / hn : 0.0);
+        double2 h0 = h[0];
+        for (int i = 0; i < j; ++i) {
+            const double2 h1 = h[i + 1], c = cs[i], s = sn[i];
+            // [h0; h1] <- [conj(c) h0 + conj(s) h1; -s h0 + c h1]
+            const double2 a = make_double2(c.x * h0.x + c.y * h0.y + s.x * h1.x + s.y * h1.y,
+                                           c.x * h0.y - c.y * h0.x + s.x * h1.y - s.y * h1.x);
+            const double2 b = make_double2(-(s.x * h0.x - s.y * h0.y) + (c.x * h1.x - c.y * h1.y),
+                                           -(s.x * h0.y + s.y * h0.x) + (c.x * h1.y + c.y * h1.x));
+            h[i] = a;
+            h0 = b;
+        }
+        const double r = sqrt(h0.x * h0.x + h0.y * h0.y + hn * hn);
+        const double2 c = r > 0 ? make_double2(h0.x / r, h0.y / r) : make_double2(1, 0);
+        const double2 s = r > 0 ? make_double2(hn / r, 0) : make_double2(0, 0);
+        st.cs[j] = c;
+        st.sn[j] = s;
+        h[j] = make_double2(r, 0);
+        st.H[(j + 1) * ldh + j] = make_double2(0, 0);
+        const double2 ej = st.e[j];
+        const double2 en = make_double2(-(s.x * ej.x - s.y * ej.y), -(s.x * ej.y + s.y * ej.x));
+        st.e[j + 1] = en;
+        st.e[j] = make_double2(c.x * ej.x + c.y * ej.y, c.x * ej.y - c.y * ej.x);
+        *st.res = sqrt(en.x * en.x + en.y * en.y);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i <= j; i += blockDim.x) st.H[i * ldh + j] = h[i];
 }
 
-// back substitution H(0:k, 0:k) y = e(0:k)
+// The second Gram-Schmidt subtraction of Arnoldi step j, w -= sum_{i<=j} V_i h_i, with the norm of the
+// result: each block adds up its slice's squares, the last block sums the blocks in order and does
+// the step's Givens update.
+__global__ void __launch_bounds__(LS_RED_THREADS) k_sub_norm_givens(const double2 *__restrict__ V, size_t ldv,
+                                                                    const double2 *__restrict__ h, double2 *w, long long N,
+                                                                    double2 *partial, GmresState st, int j, int ldh)
+{
+    extern __shared__ double2 hs[];  // 3 (j + 1) elements
+    __shared__ double red[LS_RED_THREADS / 32];
+    const int cnt = j + 1;
+    for (int i = threadIdx.x; i < cnt; i += blockDim.x) hs[i] = h[i];
+    __syncthreads();
+    double s = 0;
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < N; t += (long long)gridDim.x * blockDim.x) {
+        const double2 v = sub_at(V, ldv, cnt, hs, (const double2 *)w, t);
+        w[t] = v;
+        s = fma(v.x, v.x, fma(v.y, v.y, s));
+    }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double a = 0;
+        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) a += red[q];
+        partial[blockIdx.x] = make_double2(a, 0);
+    }
+    if (!last_block(st.ticket)) return;
+    if (threadIdx.x < 32) {
+        const double2 t = warp_total(partial, gridDim.x, 0);
+        if (threadIdx.x == 0) red[0] = t.x;
+    }
+    __syncthreads();
+    givens_step(st, j, ldh, red[0], hs);
+}
+
+// back substitution H(0:k, 0:k) y = e(0:k), column by column: the block's threads keep the right-hand
+// side in shared memory and take off each solved unknown's column
 __global__ void k_gmres_solve(GmresState st, int k, int ldh)
 {
-    if (threadIdx.x != 0) return;
+    extern __shared__ double2 acc[];  // k elements
+    for (int t = threadIdx.x; t < k; t += blockDim.x) acc[t] = st.e[t];
+    __syncthreads();
     for (int i = k - 1; i >= 0; --i) {
-        double2 acc = st.e[i];
-        for (int t = i + 1; t < k; ++t) {
-            double2 h = st.H[i * ldh + t], yt = st.y[t];
-            acc.x -= h.x * yt.x - h.y * yt.y;
-            acc.y -= h.x * yt.y + h.y * yt.x;
-        }
-        double2 d = st.H[i * ldh + i];
-        double dd = d.x * d.x + d.y * d.y;
-        st.y[i] = make_double2((acc.x * d.x + acc.y * d.y) / dd, (acc.y * d.x - acc.x * d.y) / dd);
+        const double2 d = st.H[i * ldh + i], e = acc[i];
+        const double2 h0 = (int)threadIdx.x < i ? st.H[(int)threadIdx.x * ldh + i] : make_double2(0, 0);
+        const double dd = d.x * d.x + d.y * d.y;
+        const double2 y = make_double2((e.x * d.x + e.y * d.y) / dd, (e.y * d.x - e.x * d.y) / dd);
+        if (threadIdx.x == 0) st.y[i] = y;
+        for (int t = threadIdx.x; t < i; t += blockDim.x)
+            acc[t] = axpy_acc<-1>(acc[t], t == (int)threadIdx.x ? h0 : st.H[t * ldh + i], y);
+        __syncthreads();
     }
 }
 
@@ -424,7 +575,7 @@ struct Solver {
     int restart;
     LsWork W;
     cudaStream_t st;
-    int grid_elem;
+    int grid_elem, grid_norm;  // grid_norm <= (restart + 1) LS_RED_BLOCKS: its partial sums
     std::vector<cudaGraphExec_t> *graphs = nullptr;  // the cached workspace's iteration graphs, or none
     cudaStream_t cap_stream = nullptr;               // where those graphs are captured
 
@@ -475,19 +626,23 @@ struct Solver {
     conv_status enqueue_iteration(int j, int ldh)
     {
         double2 *vj = W.V + (size_t)j * N, *vn = W.V + (size_t)(j + 1) * N;
-        conv_status rc = matvec(vj, W.w);
+        const bool f32 = p->prec != CONV_P_FP64;
+        conv_status rc = f32 ? conv_apply_axpby(p, W.v32, W.m32, W.w32, batch, kappa2, 0.0, 1.0, W.cws, st) : matvec(vj, W.w);
         if (rc != CONV_OK) return rc;
-        // CGS with one re-orthogonalisation: h = V^H w; w -= V h; h2 = V^H w; w -= V h2
-        for (int pass = 0; pass < 2; ++pass) {
-            k_multidot<<<LS_RED_BLOCKS, LS_RED_THREADS, 0, st>>>(W.V, N, j + 1, W.w, N, W.partial);
-            k_finalize_dots<<<j + 1, 32, 0, st>>>(W.partial, LS_RED_BLOCKS, j + 1, W.gs.hcol, pass);
-            // subtract with this pass's coefficients only: recompute them into y scratch
-            k_finalize_dots<<<j + 1, 32, 0, st>>>(W.partial, LS_RED_BLOCKS, j + 1, W.gs.y, 0);
-            k_sub_combination<<<grid_elem, 256, (j + 1) * sizeof(double2), st>>>(W.V, N, j + 1, W.gs.y, W.w, N);
+        // CGS with one re-orthogonalisation: y = V^H w; w -= V y, twice; h is the two y's sum.  The FP32
+        // matvec's result is read in place of w by the first pass, its input was written by the
+        // scaling of the step before.
+        const size_t sh = (size_t)(j + 1) * sizeof(double2);
+        if (f32) {
+            k_gs_dots<<<LS_RED_BLOCKS, LS_RED_THREADS, 0, st>>>(W.V, N, j + 1, W.w32, N, W.partial, W.gs.hcol, 0, W.gs.y, W.gs.ticket);
+            k_sub_combination<<<grid_elem, 256, sh, st>>>(W.V, N, j + 1, W.gs.y, W.w32, W.w, N);
+        } else {
+            k_gs_dots<<<LS_RED_BLOCKS, LS_RED_THREADS, 0, st>>>(W.V, N, j + 1, W.w, N, W.partial, W.gs.hcol, 0, W.gs.y, W.gs.ticket);
+            k_sub_combination<<<grid_elem, 256, sh, st>>>(W.V, N, j + 1, W.gs.y, W.w, W.w, N);
         }
-        norm2(W.w);
-        k_scale_by_invnorm<<<grid_elem, 256, 0, st>>>(W.w, vn, W.gs.nrm2, N);
-        k_gmres_givens<<<1, 32, 0, st>>>(W.gs, j, ldh);
+        k_gs_dots<<<LS_RED_BLOCKS, LS_RED_THREADS, 0, st>>>(W.V, N, j + 1, W.w, N, W.partial, W.gs.hcol, 1, W.gs.y, W.gs.ticket);
+        k_sub_norm_givens<<<grid_norm, LS_RED_THREADS, 3 * sh, st>>>(W.V, N, W.gs.y, W.w, N, W.partial, W.gs, j, ldh);
+        k_scale_by_invnorm<<<grid_elem, 256, 0, st>>>(W.w, vn, W.gs.nrm2, N, f32 ? W.v32 : nullptr);
         WSC_CUDA(cudaMemcpyAsync(W.host_res, W.gs.res, sizeof(double), cudaMemcpyDeviceToHost, st));
         return CONV_OK;
     }
@@ -550,7 +705,7 @@ struct Solver {
             if (!(beta == beta)) return fail(CONV_ENONFINITE, "GMRES residual is not finite");
             if (beta <= tol_abs) return CONV_OK;
             if (iters >= maxit) return fail(CONV_ENOTCONVERGED, "GMRES reached its iteration limit");
-            k_scale_by_invnorm<<<grid_elem, 256, 0, st>>>(W.r, W.V, W.gs.nrm2, N);
+            k_scale_by_invnorm<<<grid_elem, 256, 0, st>>>(W.r, W.V, W.gs.nrm2, N, p->prec != CONV_P_FP64 ? W.v32 : nullptr);
             ++cycles;
             int j = 0;
             bool reached = false;
@@ -568,7 +723,7 @@ struct Solver {
                     break;
                 }
             }
-            k_gmres_solve<<<1, 32, 0, st>>>(W.gs, j, ldh);
+            k_gmres_solve<<<1, 64, std::max(j, 1) * sizeof(double2), st>>>(W.gs, j, ldh);
             k_add_combination<<<grid_elem, 256, std::max(j, 1) * sizeof(double2), st>>>(W.V, N, j, W.gs.y, z, N);
             WSC_CUDA(cudaGetLastError());
             if (reached && trust_estimate) return CONV_OK;
@@ -631,6 +786,7 @@ static conv_status ls_solve_impl(conv_plan_t p, const double *m, const void *f, 
     int sms = 148;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
     S.grid_elem = (int)std::min<long long>((N + 255) / 256, (long long)sms * 8);
+    S.grid_norm = (int)std::min<long long>((N + 255) / 256, 2LL * LS_RED_BLOCKS);
     // workspace: the plan's cached one when free (reallocated if it does not match), else a
     // private one
     const bool mixed = p->prec == CONV_P_FP32;
@@ -681,6 +837,7 @@ static conv_status ls_solve_impl(conv_plan_t p, const double *m, const void *f, 
         free_work(S.W);
         return fail(CONV_ENOMEM, "ls_solve workspace allocation failed");
     }
+    WSC_CUDA(cudaMemsetAsync(S.W.gs.ticket, 0, sizeof(unsigned), st));
     if (p->prec == CONV_P_FP32) k_d2f<<<S.grid_elem, 256, 0, st>>>(m, S.W.m32, NN);
 
     const double2 *fb = reinterpret_cast<const double2 *>(f);
