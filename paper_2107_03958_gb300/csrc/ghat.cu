@@ -85,10 +85,14 @@ __device__ double pow_moment_cc(double gamma, double s, double a)
 // tabulates them once per plan (tab: per node u, weight, Re H0, Im H0), so only J0 is evaluated
 // here.
 // Entries in the resonance band |s - kappa| < HELM_BAND kappa, k1 >= k2 (k_ghat leaves them, and
-// their mirrors, to this kernel): one warp per entry, the lanes taking every 32nd node of the
-// table, the partial sums combined by shuffles.  Block k2 covers the band's k1 range of row k2.
-__global__ void k_ghat_band(double kappa, double scale, double b, double a, int h, double *out,
-                            const double *__restrict__ tab, int nodes)
+// their mirrors, to this kernel): one block per entry, the threads taking every 256th node of the table,
+// their sums combined by shuffles and then over the warps.  Blocks (k2, y): the band's k1 range of row k2
+// from its y-th entry in steps of the grid's height; only rows that meet the band are launched, since
+// every warp pays FP64 square roots to find its range.  The band holds few entries (31 at kappa = 33) of
+// thousands of nodes each, so a warp per entry left most of the chip idle (n = 256, kappa = 33:
+// 201 us; a block per entry 54 us).
+__global__ void __launch_bounds__(256) k_ghat_band(double kappa, double scale, double b, double a, int h, double *out,
+                                                   const double *__restrict__ tab, int nodes)
 {
     const int k2 = blockIdx.x;
     if (k2 >= h) return;
@@ -96,14 +100,15 @@ __global__ void k_ghat_band(double kappa, double scale, double b, double a, int 
     const double rlo = kr * (1.0 - HELM_BAND), rhi = kr * (1.0 + HELM_BAND), k2d = (double)k2;
     const int lo = max(k2, (int)floor(sqrt(fmax(0.0, rlo * rlo - k2d * k2d))) - 1);
     const int hi = min(h - 1, (int)ceil(sqrt(fmax(0.0, rhi * rhi - k2d * k2d))) + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int k1 = lo + warp; k1 <= hi; k1 += nw) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ double2 red[8];
+    for (int k1 = lo + blockIdx.y; k1 <= hi; k1 += gridDim.y) {
         // the same test as k_ghat's, on the same arithmetic
         const double km = hypot((double)k1, k2d);
         const double s = 2.0 * M_PI * km / b;
         if (km == 0.0 || !(fabs(s - kappa) < HELM_BAND * kappa)) continue;
         double sr = 0.0, si = 0.0;
-        for (int i = lane; i < nodes; i += 32) {
+        for (int i = threadIdx.x; i < nodes; i += blockDim.x) {
             const double u = tab[4 * i], u4 = u * u * u * u;
             const double w = tab[4 * i + 1] * j0(s * a * u4) * u4 * u * u * u;
             sr += w * tab[4 * i + 2];
@@ -114,12 +119,20 @@ __global__ void k_ghat_band(double kappa, double scale, double b, double a, int 
             sr += __shfl_xor_sync(0xffffffffu, sr, o);
             si += __shfl_xor_sync(0xffffffffu, si, o);
         }
-        if (lane == 0) {
+        if (lane == 0) red[warp] = make_double2(sr, si);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            sr = si = 0.0;
+            for (int q = 0; q < 8; ++q) {
+                sr += red[q].x;
+                si += red[q].y;
+            }
             const double c = 2.0 * M_PI * a * a;
             const long long idx = (long long)k2 * h + k1, mirror = (long long)k1 * h + k2;
             out[2 * idx] = out[2 * mirror] = scale * (-c * si);
             out[2 * idx + 1] = out[2 * mirror + 1] = scale * (c * sr);
         }
+        __syncthreads();
     }
 }
 
@@ -146,10 +159,25 @@ __global__ void k_helm_band_table(double *__restrict__ tab, int P, double ka)
 __global__ void k_ghat(int family, double gamma, double kappa, double scale, double b, double a,
                        int h, double *out, double4 hka)
 {
-    const long long N = (long long)h * h;
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < N;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int k2 = (int)(idx / h), k1 = (int)(idx - (long long)k2 * h);
+    // work items: every entry of the non-radial table; for a radial one the triangle k1 >= k2, folded into
+    // rows of equal length (row r holds k2 = r from k1 = r on, then k2 = h - 1 - r), so that no lane of
+    // a warp waits through its neighbours' Bessel functions for a mirrored entry
+    const bool radial = family != CONV_K_DX1LOG;
+    const int width = radial ? h + 1 : h;
+    const long long N = radial ? (long long)((h + 1) / 2) * width : (long long)h * h;
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < N; t += (long long)gridDim.x * blockDim.x) {
+        int k2 = (int)(t / width), k1 = (int)(t - (long long)k2 * width);
+        if (radial) {
+            if (k1 < h - k2) {
+                k1 += k2;
+            } else {  // h - k2 entries of row k2 came first; k2 + 1 entries of row h - 1 - k2 follow
+                const int i = k1 - (h - k2);
+                if (2 * k2 == h - 1) continue;  // the middle row has no partner
+                k2 = h - 1 - k2;
+                k1 = k2 + i;
+            }
+        }
+        const long long idx = (long long)k2 * h + k1;
         const double km = hypot((double)k1, (double)k2);
         const double s = 2.0 * M_PI * km / b, z = s * a;
         if (family == CONV_K_DX1LOG) {
@@ -159,7 +187,6 @@ __global__ void k_ghat(int family, double gamma, double kappa, double scale, dou
             continue;
         }
         // ghat depends on |k| only: each entry with k1 >= k2 also fills its mirror [k1][k2]
-        if (k1 < k2) continue;
         const long long mirror = (long long)k1 * h + k2;
         if (family == CONV_K_LOG) {
             double G;
@@ -309,8 +336,10 @@ conv_status build_ghat(conv_plan_s *p)
         int blocks = (int)std::min<long long>((N + 255) / 256, 152LL * 16);
         k_ghat<<<blocks, 256, 0, st>>>(p->kern.family, p->kern.gamma, p->kern.kappa, scale, p->b, p->a, hb,
                                        p->ghat_paper, hka);
-        if (htab)  // the resonance band's entries
-            k_ghat_band<<<hb, 256, 0, st>>>(p->kern.kappa, scale, p->b, p->a, hb, p->ghat_paper, htab, hnodes);
+        // the resonance band's entries: rows k2 <= k1, so up to its outer radius over sqrt 2
+        const int band_rows = std::min(hb, (int)(p->kern.kappa * p->b / (2.0 * M_PI) * (1.0 + HELM_BAND) / std::sqrt(2.0)) + 3);
+        if (htab)
+            k_ghat_band<<<dim3(band_rows, 16), 256, 0, st>>>(p->kern.kappa, scale, p->b, p->a, hb, p->ghat_paper, htab, hnodes);
         if (htab) cudaFreeAsync(htab, st);  // in stream order, after the kernels that read it
         WSC_CUDA(cudaGetLastError());
     } else {

@@ -144,17 +144,17 @@ static bool factorize(int L, int E, FFTDesc &d, bool radix16 = false)
 // w = exp(-2 pi i / (Ns R)), in long double.
 void stage_twiddles(const FFTDesc &d, std::vector<double> &re_im)
 {
-    const long double PI_L = 3.141592653589793238462643383279502884L;
+    std::vector<double> re, im;
+    unit_roots(d.L, [](long double x) { return (double)x; }, re, im);
     re_im.assign(2 * (size_t)d.tw_len, 0.0);
     for (int s = 0; s < d.nst; ++s) {
         const long long Ns = d.Ns[s], NR = Ns * d.R[s];
         for (int m = 0; m < tw_blocks(d.R[s]); ++m)
             for (long long k = 0; k < Ns; ++k) {
-                const long long e = ((1LL << m) * k) % NR;
-                const long double ang = 2.0L * PI_L * (long double)e / (long double)NR;
+                const size_t e = (size_t)(((1LL << m) * k) % NR * (d.L / NR));
                 const size_t i = (size_t)d.toff[s] + (size_t)m * Ns + (size_t)k;
-                re_im[2 * i] = (double)cosl(ang);
-                re_im[2 * i + 1] = (double)-sinl(ang);
+                re_im[2 * i] = re[e];
+                re_im[2 * i + 1] = im[e];
             }
     }
 }
@@ -468,6 +468,7 @@ static bool configure(conv_plan_s *p, const Candidate &c, int smem_optin, int sm
         S.tma = tma;
         S.stage = (int)(sb / esz);
         S.smem = pass_smem(tws ? twb : 0, pb, sb, G);
+        S.smem_group = pass_smem(0, pb, sb, 2) - pass_smem(0, pb, sb, 1);
         int bps = 1;
         if (fused)
             WSC_DISPATCH_FUSED(p->prec, E, ed, tws, bps = (blocks_per_sm_fused<T_, E_, ED_, W_>(tpt * G, S.smem)));
@@ -527,6 +528,7 @@ static bool configure(conv_plan_s *p, const Candidate &c, int smem_optin, int sm
         C = I = R;  // the plain kernels share one twiddle option and shape
     }
     p->r2c_split = split;
+    p->sms = sms;
     p->elems = E;
     p->tws = R.tws;
     p->fft = d;

@@ -61,39 +61,11 @@ static bool fixed_factor(int L, FixedDesc &d)
     return true;
 }
 
-// exp(-2 pi i t / L) for every t, from the first octant
-static void unit_roots(int L, std::vector<long double> &re, std::vector<long double> &im)
+// v / 2^shift, rounded, as h 2^32 + l with l signed and its negation in range
+static void split_scaled(long long v, int shift, int &h, int &l)
 {
-    const long double PI_L = 3.141592653589793238462643383279502884L;
-    re.resize(L);
-    im.resize(L);
-    auto put = [&](long long t, long double c, long double s) {  // angle 2 pi t / L: (c, -s)
-        t = ((t % L) + L) % L;
-        re[t] = c;
-        im[t] = -s;
-    };
-    if (L % 8 == 0) {
-        for (int t = 0; t <= L / 8; ++t) {
-            const long double x = 2.0L * PI_L * (long double)t / (long double)L, c = cosl(x), s = sinl(x);
-            for (int q = 0; q < 4; ++q) {  // rotations by a quarter turn of t and of its mirror L/4 - t
-                const long double cq[4] = {c, -s, -c, s}, sq[4] = {s, c, -s, -c};
-                put((long long)q * (L / 4) + t, cq[q], sq[q]);
-                const long double cm[4] = {s, -c, -s, c}, sm[4] = {c, s, -c, -s};
-                put((long long)q * (L / 4) + L / 4 - t, cm[q], sm[q]);
-            }
-        }
-    } else {
-        for (int t = 0; t < L; ++t) {
-            const long double x = 2.0L * PI_L * (long double)t / (long double)L;
-            put(t, cosl(x), sinl(x));
-        }
-    }
-}
-
-static void split_scaled(long double w, int bits, int &h, int &l)
-{
-    long long v = llroundl(ldexpl(w, bits));
-    if ((int)(unsigned)(unsigned long long)v == INT32_MIN) ++v;  // its negation has to fit too
+    if (shift) v = (v + (1LL << (shift - 1))) >> shift;
+    if ((int)(unsigned)(unsigned long long)v == INT32_MIN) ++v;
     l = (int)(unsigned)(unsigned long long)v;
     h = (int)((v - l) / (1LL << 32));
 }
@@ -101,8 +73,8 @@ static void split_scaled(long double w, int bits, int &h, int &l)
 // Twiddle copies of every stage (FixedDesc), as (re h, re l, im h, im l)
 void fixed_twiddles(const FixedDesc &d, std::vector<int> &tab)
 {
-    std::vector<long double> re, im;
-    unit_roots(d.L, re, im);
+    std::vector<long long> re, im;
+    unit_roots(d.L, [](long double x) { return (long long)llroundl(ldexpl(x, 62)); }, re, im);
     tab.assign(4 * (size_t)d.tw_len, 0);
     for (int s = 1; s < d.nst; ++s) {
         const int R = d.R[s], Ns = d.Ns[s];
@@ -112,8 +84,8 @@ void fixed_twiddles(const FixedDesc &d, std::vector<int> &tab)
                 for (int k = 0; k < (d.L == 8192 && R == 2 ? d.L / 4 : Ns); ++k) {
                     const size_t t = (size_t)(((long long)q * k * step) % d.L);
                     int *e = &tab[4 * ((size_t)d.toff[s] + ((size_t)v * (R - 1) + q - 1) * Ns + k)];
-                    split_scaled(re[t], 62 - v, e[0], e[1]);
-                    split_scaled(im[t], 62 - v, e[2], e[3]);
+                    split_scaled(re[t], v, e[0], e[1]);
+                    split_scaled(im[t], v, e[2], e[3]);
                 }
     }
 }
@@ -160,7 +132,7 @@ bool fixed_configure(conv_plan_s *p, int smem_optin, int sms)
         else p->cols.groups = std::min(S.groups, two);
     }
     p->fixed_desc = d;
-    p->fixed_sms = sms;
+    p->sms = sms;
     p->fixed = p->fused = true;
     p->elems = 16;
     p->tws = false;

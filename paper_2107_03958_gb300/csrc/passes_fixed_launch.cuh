@@ -74,8 +74,8 @@ conv_status run_fixed(conv_plan_s *p, const void *u, const void *mask, void *out
     // groups per CTA: as many as fit, fewer when the work items would not reach every SM
     auto launch = [&](auto kern, const LaunchShape &S, int nbuf, int units) {
         a.units = units;
-        const int G = std::max(1, std::min(S.groups, (units + p->fixed_sms - 1) / p->fixed_sms));
-        const long long need = (units + G - 1) / G, most = (long long)p->fixed_sms * (S.groups / G);
+        const int G = std::max(1, std::min(S.groups, (units + p->sms - 1) / p->sms));
+        const long long need = (units + G - 1) / G, most = (long long)p->sms * (S.groups / G);
         const size_t smem = ((size_t)fixed_padded(L) * (LL ? nbuf : 2) * sizeof(c64) + FIXED_SLOTS * sizeof(unsigned)) * G +
                             (LL ? fixed_tw_smem(LL) * sizeof(int4) : 0);
         kern<<<(unsigned)std::min(need, most), S.tpt * G, smem, st>>>(a);

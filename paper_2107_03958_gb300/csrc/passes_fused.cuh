@@ -744,9 +744,19 @@ conv_status run_fused(conv_plan_s *p, const void *u, const void *mask, void *out
     a.alpha = cmk<V>((T)(are * sc), (T)(aim * sc));
     a.beta = (T)beta;
     const LaunchShape &R = p->rows, &C = p->cols, &I = p->inv;
-    auto grid = [&](const LaunchShape &S, int units) {
-        long long need = (units + S.groups - 1) / S.groups;
-        return (unsigned)std::min<long long>(need, (long long)S.max_ctas);
+    // Groups per CTA: as many as the shape holds, unless fewer than half the SMs would then get a CTA:
+    // one small density's rows run faster spread over the chip (C2C batch 1, passes 1 / 2 / 3:
+    // n = 512, 64 CTAs of 8 groups -> 128 of 4, 16.4 / 12.5 / 12.3 -> 12.8 / 10.8 / 10.2 us; n = 256 13.7 / 8.3 / 10.2 ->
+    // 12.2 / 8.8 / 8.2 us), while at 128 CTAs of 8 groups (batch 8 of n = 256) 147 of 7 gain nothing
+    struct Geo {
+        unsigned grid, threads;
+        size_t smem;
+    };
+    auto geo = [&](const LaunchShape &S, int units) {
+        const bool few = (units + S.groups - 1) / S.groups < p->sms / 2;
+        const int G = few ? (units + p->sms - 1) / p->sms : S.groups;
+        const long long need = (units + G - 1) / G, most = (long long)S.max_ctas * (S.groups / G);
+        return Geo{(unsigned)std::min(need, most), (unsigned)(S.tpt * G), S.smem - S.smem_group * (S.groups - G)};
     };
     // prefetch needs the staged runs to start on 16 bytes (bulk copies, 16-byte cp.async) or on
     // their element size (8-byte cp.async), and bulk copy lengths that are multiples of 16
@@ -764,13 +774,15 @@ conv_status run_fused(conv_plan_s *p, const void *u, const void *mask, void *out
 #define WSC_TARGS(T_, E_, ED_) T_, E_, ED_
 #define WSC_LAUNCH(S, K, TA)                                                                   \
     do {                                                                                      \
-        if ((S).tws) K<WSC_TARGS TA, true><<<grid(S, a.units), (S).tpt * (S).groups, (S).smem, st>>>(a);  \
-        else K<WSC_TARGS TA, false><<<grid(S, a.units), (S).tpt * (S).groups, (S).smem, st>>>(a);      \
+        const Geo g_ = geo(S, a.units);                                                       \
+        if ((S).tws) K<WSC_TARGS TA, true><<<g_.grid, g_.threads, g_.smem, st>>>(a);          \
+        else K<WSC_TARGS TA, false><<<g_.grid, g_.threads, g_.smem, st>>>(a);                 \
     } while (0)
 #define WSC_LAUNCH2(S, K, TA, X)                                                                  \
     do {                                                                                         \
-        if ((S).tws) K<WSC_TARGS TA, true, X><<<grid(S, a.units), (S).tpt * (S).groups, (S).smem, st>>>(a); \
-        else K<WSC_TARGS TA, false, X><<<grid(S, a.units), (S).tpt * (S).groups, (S).smem, st>>>(a);     \
+        const Geo g_ = geo(S, a.units);                                                          \
+        if ((S).tws) K<WSC_TARGS TA, true, X><<<g_.grid, g_.threads, g_.smem, st>>>(a);          \
+        else K<WSC_TARGS TA, false, X><<<g_.grid, g_.threads, g_.smem, st>>>(a);                 \
     } while (0)
     // kernels with a ping-pong variant: launched with it when the pass's shape holds two buffers
 #define WSC_LAUNCH_PP(S, K)                                      \

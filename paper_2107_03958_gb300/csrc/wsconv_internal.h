@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <array>
+#include <cmath>
 #include <string>
 #include <vector>
 
@@ -97,6 +98,7 @@ struct LaunchShape {
     int tpt;       // threads per transform
     int groups;    // transforms per CTA
     size_t smem;   // dynamic shared memory bytes
+    size_t smem_group;  // fused passes: the part of it that each group adds
     int max_ctas;  // persistent grid size (CTAs resident at once)
     int stage;     // fused passes: elements of each group's prefetch staging area (0: no prefetch)
     bool tws;      // twiddle table in shared memory
@@ -131,7 +133,7 @@ struct conv_plan_s {
     bool fused; // passes on the fused transform (global-memory first/last stages)
     bool fixed = false;                      // FP64 passes in 64-bit fixed point (passes_fixed.cuh)
     wsc::FixedDesc fixed_desc{};
-    int fixed_sms = 0;                       // SMs the fixed-point passes are spread over
+    int sms = 0;                             // SMs the passes are spread over
     bool long_lines = false;                 // lines beyond one CTA: four-step FP64 pipeline (fsmask.cu)
     wsc::LongLines *longl = nullptr;
     // conv_apply_kernels: for the duration of one launch, each density's multiplier table
@@ -188,6 +190,36 @@ conv_status set_all_attrs_fixed(int smem);
 conv_status launch_fixed(conv_plan_s *p, const void *u, const void *mask, void *out, int batch, double are,
                          double aim, double beta, void *ws, cudaStream_t st);
 void fixed_twiddles(const FixedDesc &d, std::vector<int> &tab);
+// exp(-2 pi i t / L) = (re[t], im[t]), t < L.  conv(x) turns a long double cosine or sine into T and is called,
+// like the two functions, on the first octant (quadrant, half) alone; the rest are its values with
+// signs and places exchanged.  (A plan's tables took a long double pair per entry, most of a small
+// plan's build where long double is software arithmetic.)
+template <class T, class F> void unit_roots(int L, F conv, std::vector<T> &re, std::vector<T> &im)
+{
+    const long double PI_L = 3.141592653589793238462643383279502884L;
+    re.resize(L);
+    im.resize(L);
+    const int fold = L % 8 == 0 ? 8 : (L % 4 == 0 ? 4 : (L % 2 == 0 ? 2 : 1));
+    for (int t = 0; t <= (fold > 1 ? L / fold : L - 1); ++t) {
+        const long double x = 2.0L * PI_L * (long double)t / (long double)L;
+        const T c = conv(cosl(x)), s = conv(sinl(x));
+        auto put = [&](int u, T cu, T su) {  // angle 2 pi u / L: (cos, sin)
+            re[u % L] = cu;
+            im[u % L] = -su;
+        };
+        if (fold <= 2) {
+            put(t, c, s);
+            if (fold == 2) put(t + L / 2, -c, -s);
+            continue;
+        }
+        const T cq[4] = {c, -s, -c, s}, sq[4] = {s, c, -s, -c};  // quarter turns
+        for (int q = 0; q < 4; ++q) put(q * (L / 4) + t, cq[q], sq[q]);
+        if (fold == 8) {
+            const T cm[4] = {s, -c, -s, c}, sm[4] = {c, s, -c, -s};  // and of the mirror L/4 - t
+            for (int q = 0; q < 4; ++q) put(q * (L / 4) + L / 4 - t, cm[q], sm[q]);
+        }
+    }
+}
 // ghat.cu
 conv_status build_ghat(conv_plan_s *p);
 conv_status copy_ghat(conv_plan_s *p, const conv_plan_s *src);  // src's FP64 tables, no recomputation
