@@ -82,6 +82,7 @@ __device__ __forceinline__ typename cvec<T>::t *setup_smem(const PassArgs<T> &a,
     } else {
         twp = a.tw;
     }
+    pdl_wait();  // nothing a predecessor wrote has been read yet
     return base + (size_t)g * padded_len<T>(a.M);
 }
 

@@ -368,6 +368,7 @@ __device__ __forceinline__ c64 *fixed_smem(const FixedArgs &a, int g, int G, int
     for (int i = threadIdx.x; i < ntw; i += blockDim.x) t[i] = __ldg(a.tw + i);
     for (int i = threadIdx.x; i < FIXED_SLOTS * G; i += blockDim.x) slots[i] = 0;
     __syncthreads();
+    pdl_wait();
     tws = t;
     return base + (size_t)per * g;
 }
@@ -376,6 +377,7 @@ __device__ __forceinline__ c64 *fixed_smem(const FixedArgs &a, int g, int G, int
 __device__ __forceinline__ bool fixed_gives_up(const FixedArgs &a)
 {
     if (!a.give_up) return false;
+    pdl_wait();
     if (threadIdx.x == 0) atomicExch(a.err, (int)CONV_ETIMEOUT);
     return true;
 }

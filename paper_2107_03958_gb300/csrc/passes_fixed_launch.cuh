@@ -71,6 +71,7 @@ conv_status run_fixed(conv_plan_s *p, const void *u, const void *mask, void *out
     a.alpha = make_double2(are * sc, aim * sc);
     fixed_alpha(a.alpha.x, a.alpha.y, a.ah, a.al, a.ae);
     a.beta = beta;
+    const bool may_early = may_launch_early(st);
     // groups per CTA: as many as fit, fewer when the work items would not reach every SM
     auto launch = [&](auto kern, const LaunchShape &S, int nbuf, int units) {
         a.units = units;
@@ -78,7 +79,7 @@ conv_status run_fixed(conv_plan_s *p, const void *u, const void *mask, void *out
         const long long need = (units + G - 1) / G, most = (long long)p->sms * (S.groups / G);
         const size_t smem = ((size_t)fixed_padded(L) * (LL ? nbuf : 2) * sizeof(c64) + FIXED_SLOTS * sizeof(unsigned)) * G +
                             (LL ? fixed_tw_smem(LL) * sizeof(int4) : 0);
-        kern<<<(unsigned)std::min(need, most), S.tpt * G, smem, st>>>(a);
+        launch_pass(kern, may_early && need <= p->sms, (unsigned)std::min(need, most), (unsigned)(S.tpt * G), smem, st, a);
     };
     cudaEvent_t *ev = timing_slot(p);
     if (ev) cudaEventRecord(ev[0], st);

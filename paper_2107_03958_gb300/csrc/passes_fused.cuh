@@ -751,12 +751,14 @@ conv_status run_fused(conv_plan_s *p, const void *u, const void *mask, void *out
     struct Geo {
         unsigned grid, threads;
         size_t smem;
+        bool early;
     };
+    const bool may_early = may_launch_early(st);
     auto geo = [&](const LaunchShape &S, int units) {
         const bool few = (units + S.groups - 1) / S.groups < p->sms / 2;
         const int G = few ? (units + p->sms - 1) / p->sms : S.groups;
         const long long need = (units + G - 1) / G, most = (long long)S.max_ctas * (S.groups / G);
-        return Geo{(unsigned)std::min(need, most), (unsigned)(S.tpt * G), S.smem - S.smem_group * (S.groups - G)};
+        return Geo{(unsigned)std::min(need, most), (unsigned)(S.tpt * G), S.smem - S.smem_group * (S.groups - G), may_early && need <= p->sms};
     };
     // prefetch needs the staged runs to start on 16 bytes (bulk copies, 16-byte cp.async) or on
     // their element size (8-byte cp.async), and bulk copy lengths that are multiples of 16
@@ -775,14 +777,14 @@ conv_status run_fused(conv_plan_s *p, const void *u, const void *mask, void *out
 #define WSC_LAUNCH(S, K, TA)                                                                   \
     do {                                                                                      \
         const Geo g_ = geo(S, a.units);                                                       \
-        if ((S).tws) K<WSC_TARGS TA, true><<<g_.grid, g_.threads, g_.smem, st>>>(a);          \
-        else K<WSC_TARGS TA, false><<<g_.grid, g_.threads, g_.smem, st>>>(a);                 \
+        if ((S).tws) launch_pass(K<WSC_TARGS TA, true>, g_.early, g_.grid, g_.threads, g_.smem, st, a);  \
+        else launch_pass(K<WSC_TARGS TA, false>, g_.early, g_.grid, g_.threads, g_.smem, st, a);         \
     } while (0)
 #define WSC_LAUNCH2(S, K, TA, X)                                                                  \
     do {                                                                                         \
         const Geo g_ = geo(S, a.units);                                                          \
-        if ((S).tws) K<WSC_TARGS TA, true, X><<<g_.grid, g_.threads, g_.smem, st>>>(a);          \
-        else K<WSC_TARGS TA, false, X><<<g_.grid, g_.threads, g_.smem, st>>>(a);                 \
+        if ((S).tws) launch_pass(K<WSC_TARGS TA, true, X>, g_.early, g_.grid, g_.threads, g_.smem, st, a);  \
+        else launch_pass(K<WSC_TARGS TA, false, X>, g_.early, g_.grid, g_.threads, g_.smem, st, a);         \
     } while (0)
     // kernels with a ping-pong variant: launched with it when the pass's shape holds two buffers
 #define WSC_LAUNCH_PP(S, K)                                      \

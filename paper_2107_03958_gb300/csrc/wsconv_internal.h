@@ -47,6 +47,46 @@ template <typename T, int E, int ED> struct maxt_fused {
 __host__ __device__ constexpr bool pingpong_ed(int ed, int elem_bytes) { return elem_bytes == 4 && (ed == 1012 || ed == 1013); }
 template <typename T, int ED> __host__ __device__ constexpr bool pingpong_ok() { return pingpong_ed(ED, (int)sizeof(T)); }
 
+// A pass kernel's launch.  early: programmatic dependent launch, so that the launch and the kernel's
+// set-up (shared memory, twiddle copies, which only read the plan's tables) overlap the tail of its
+// predecessor on the stream.  Every pass kernel calls pdl_wait() before it touches anything its
+// predecessors wrote or read, on every path; what follows it on the stream then also follows them.
+// Used where a launch's CTAs all run at once (the passes of a small grid are a few microseconds each:
+// FP32 n = 64 29.9 -> 22.2 us, FP64 n = 64 31.0 -> 27.1, FP64 n = 256 batch 16 90.8 -> 84.8) and not under
+// capture (the FP64 LS step graphs at n = 512: 2.69 -> 2.81 ms a solve) or for grids of several rounds,
+// where waiting CTAs gain nothing.
+template <class... P, class... A>
+inline cudaError_t launch_pass(void (*kernel)(P...), bool early, unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+// whether launches on st may be early ones
+inline bool may_launch_early(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return cs == cudaStreamCaptureStatusNone;
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait()
+{
+    asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
+}
+#endif
+
 template <typename T, int E, bool TWS>
 conv_status run_pipeline(conv_plan_s *p, const void *u, const void *mask, void *out, int batch,
                          double are, double aim, double beta, void *ws, cudaStream_t st);
