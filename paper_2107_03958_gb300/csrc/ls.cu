@@ -647,7 +647,7 @@ struct Solver {
         return CONV_OK;
     }
 
-    // Step j as one graph launch when the workspace is the plan's: the ~17 launches of a step are
+    // Step j as one graph launch when the workspace is the plan's: the eight launches of a step are
     // captured once and replayed, so the GPU does not wait on the host's launches after every
     // residual check.  Every pointer the step uses belongs to the plan or its cached workspace.
     conv_status run_iteration(int j, int ldh)

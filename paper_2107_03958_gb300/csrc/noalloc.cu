@@ -49,6 +49,15 @@ extern "C" conv_status conv_apply_noalloc(conv_plan_t p, const void *u, const vo
     void *ws = nullptr;
     conv_status rc = check_apply(p, u, mask, out, batch, 0.0, p->noalloc_scratch, &ws);
     if (rc != CONV_OK || batch == 0) return rc;
+    // Helmholtz R2C in fixed point: where the split column pass's scratch lines do not fit behind the
+    // spectra, the passes on complex lines take the call (the spectra's room holds theirs)
+    const bool split = p->r2c_split;
+    if (p->fixed && workspace_bytes(p, batch) > WSCONV_NOALLOC_SCRATCH_BYTES) p->r2c_split = false;
+    struct Restore {
+        conv_plan_s *p;
+        bool split;
+        ~Restore() { p->r2c_split = split; }
+    } restore{p, split};
     const size_t need = workspace_bytes(p, batch);
     if (need > WSCONV_NOALLOC_SCRATCH_BYTES)
         return fail(CONV_EINVAL, "conv_apply_noalloc: this plan and batch need " + std::to_string(need) +

@@ -382,6 +382,22 @@ static int default_options(const conv_plan_s *p, int ed, int pass)
     return pass == 1 ? CFG_TWS : CFG_TWS | CFG_PF | CFG_TMA;
 }
 
+// Lengths conv_apply_multi takes in FP64: the powers of two 2^10 ... 2^13 at n = L/2, and those the
+// first fitting FP64 stage structure runs fused.  The fixed-point passes could share pass 1 at every
+// length; the call's domain is part of its interface and does not depend on which passes run.
+static bool multi_length64(const conv_plan_s *p, int smem_optin)
+{
+    if (2 * p->n == p->M && p->M >= 1024 && p->M <= 8192 && (p->M & (p->M - 1)) == 0) return true;
+    for (int E : kElems64) {
+        FFTDesc d;
+        if (E == 16 || E == 0 || p->M % E || !factorize(p->M, E, d) || p->M / E > max_threads(CONV_P_FP64, E)) continue;
+        // split R2C: pass 2 needs two buffers in one CTA
+        const size_t line = (size_t)padded_len<double>(p->M) * sizeof(double2);
+        return fused_edges(CONV_P_FP64, E, d) && (p->io != CONV_IO_R2C || pass_smem(0, 2 * line, 0, 1) <= (size_t)smem_optin);
+    }
+    return false;
+}
+
 // One launch configuration c = {E elements per thread, fused passes (1 when eligible, preferring a
 // compile-time length; 2 when eligible, runtime stage structure; 0 never),
 // options of pass 1, 2, 3 (CFG_* bits: shared-memory twiddles when they fit, prefetch when it
@@ -395,7 +411,11 @@ static bool configure(conv_plan_s *p, const Candidate &c, int smem_optin, int sm
     // FP64 lines of 32 to 8192 points (as far as two buffers fit beside each other, for the lengths
     // without kernels of their own) run in fixed point: 3.6 to 4.7 times the FP64 stages' rate from n = 256 on,
     // 1.6 times at n = 64 (n = 4096, batch 16: 125.3 -> 27.6 ms; n = 480, period 3, batch 8: 2266 -> 592 us)
-    if (p->prec == CONV_P_FP64 && E == 16) return fused_pref == 1 && fixed_configure(p, smem_optin, sms);
+    p->multi_ok = true;
+    if (p->prec == CONV_P_FP64 && E == 16) {
+        p->multi_ok = multi_length64(p, smem_optin);
+        return fused_pref == 1 && fixed_configure(p, smem_optin, sms);
+    }
     const size_t esz = p->prec == CONV_P_FP64 ? 16 : 8;
     const size_t per = (size_t)(p->prec == CONV_P_FP64 ? padded_len<double>(M) : padded_len<float>(M)) * esz;
     FFTDesc d;

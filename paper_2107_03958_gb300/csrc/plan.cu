@@ -72,8 +72,11 @@ size_t workspace_bytes(const conv_plan_s *p, int batch)
 {
     if (p->long_lines) return batch > 0 ? long_lines_ws_bytes(p) : 0;  // densities run one at a time
     const size_t esz = p->prec == CONV_P_FP64 ? 16 : 8;
-    // the split pass 2's scratch lines follow the spectra on an even element
-    const size_t scratch = p->split_scratch_elems ? p->split_scratch_elems + 1 : 0;
+    // the split pass 2's scratch lines follow the spectra on an even element; the fixed-point passes
+    // use no more of them than columns, rounded up to whole CTAs
+    size_t lines = p->split_scratch_elems;
+    if (p->fixed) lines = std::min(lines, ((size_t)batch * p->h + p->cols.groups) * p->M);
+    const size_t scratch = p->r2c_split && lines ? lines + 1 : 0;
     return batch > 0 ? (spectrum_elems(p) * (size_t)batch + scratch) * esz : 0;
 }
 
@@ -575,7 +578,7 @@ static conv_status check_multi(const conv_plan_t *plans, int count)
     for (int k = 0; k < count; ++k) {
         const conv_plan_s *q = plans[k];
         if (!q) return fail(CONV_EINVAL, "conv_apply_multi: a plan in the list is NULL");
-        if (!q->fused || q->long_lines || !(q->io == CONV_IO_R2R || q->r2c_split))
+        if (!q->fused || !q->multi_ok || q->long_lines || !(q->io == CONV_IO_R2R || q->r2c_split))
             return fail(CONV_EUNSUPPORTED, "conv_apply_multi: every plan must run the fused R2R or split R2C passes");
         if (q->timing) return fail(CONV_EINVAL, "conv_apply_multi: per-pass timing is on");
         if (q->n != p0->n || q->Mb != p0->Mb || q->M != p0->M || q->prec != p0->prec || q->compact != p0->compact ||

@@ -173,6 +173,7 @@ struct conv_plan_s {
     bool fused; // passes on the fused transform (global-memory first/last stages)
     bool fixed = false;                      // FP64 passes in 64-bit fixed point (passes_fixed.cuh)
     wsc::FixedDesc fixed_desc{};
+    bool multi_ok = true;                    // conv_apply_multi takes the plan's line length
     int sms = 0;                             // SMs the passes are spread over
     bool long_lines = false;                 // lines beyond one CTA: four-step FP64 pipeline (fsmask.cu)
     wsc::LongLines *longl = nullptr;

@@ -7,6 +7,7 @@ Tolerance: four transforms of at most 8192 points, each within 2.6e-16 of its re
 error of FP64 transforms of that length), plus the other side's: 8 x 2.6e-16, and a factor 2.5 from
 the 2-norm to the largest element: 5e-15.
 """
+import ctypes
 import math
 
 import numpy as np
@@ -14,8 +15,9 @@ import pytest
 import torch
 
 import oracle as O
-from paper_2107_03958_gb300 import inputs
-from paper_2107_03958_gb300.api import ConvPlan
+from paper_2107_03958_gb300 import _native, inputs
+from paper_2107_03958_gb300._native import ConvError
+from paper_2107_03958_gb300.api import ConvPlan, multi_workspace_bytes
 
 pytestmark = pytest.mark.gpu
 
@@ -105,3 +107,34 @@ def test_non_power_of_two_scale_and_single_spike():
     u = np.zeros((n, n))
     u[7, 53] = 0.7
     assert _err(O.conv(u, p.M, _table(p)).real, _apply(p, u)) <= TOL
+
+
+@pytest.mark.parametrize("n,period,compact,B", [(256, 3, True, 8), (60, 4, False, 80), (60, 4, False, 95)])
+def test_noalloc_without_room_for_scratch_lines(n, period, compact, B):
+    """Helmholtz R2C whose spectra fit the fixed scratch array and whose parked spectra do not: taken on
+    complex lines.  Two results, each within TOL of the exact one."""
+    plan = _plan(n, period, compact, "r2c", batch=1)
+    L = plan.info.transform_len
+    spectra = (3 * (L // 2 + 1) * n + 1) * B * 16
+    assert spectra <= 32 << 20 < plan.workspace_bytes(B)
+    u = torch.tensor(inputs.bump_sums(n, B, seed=5), device="cuda")
+    ref = plan.apply(u, workspace=torch.empty(plan.workspace_bytes(B) // 8 + 2, dtype=torch.float64, device="cuda"))
+    out = torch.full_like(ref, float("nan"))
+    st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    rc = _native.load().conv_apply_noalloc(plan.handle, ctypes.c_void_p(u.data_ptr()), None,
+                                           ctypes.c_void_p(out.data_ptr()), B, st)
+    assert rc == 0, _native.load().conv_last_error()
+    assert plan.info.r2c_split == 1
+    r, o = ref.cpu().numpy(), out.cpu().numpy()
+    assert np.max(np.abs(o - r)) <= 2 * TOL * np.max(np.abs(r))
+
+
+@pytest.mark.parametrize("n,period,compact,taken", [(64, 5, False, False), (64, 3, False, True), (512, 3, True, True),
+                                                    (100, 3, False, False), (256, 3, True, True)])
+def test_multi_takes_the_lengths_of_its_domain(n, period, compact, taken):
+    plans = [_plan(n, period, compact, "r2r") for _ in range(2)]
+    if taken:
+        assert multi_workspace_bytes(plans, 1) > 0
+    else:
+        with pytest.raises(ConvError, match="EUNSUPPORTED"):
+            multi_workspace_bytes(plans, 1)
