@@ -24,6 +24,8 @@
 // A line with an infinity or a NaN becomes all NaN (its FP64 transform would be, but for a few
 // infinities).  A line whose exponents leave the normal range is converted by scalbn.
 #pragma once
+#include <climits>
+
 #include "fft_engine.cuh"
 #include "wsconv_internal.h"
 
@@ -42,6 +44,9 @@ __device__ __forceinline__ split64 split_of(long long v)
     s.h += (int)((unsigned)s.l >> 31);
     return s;
 }
+// The same for a factor whose halves are negated: where l is INT_MIN, whose negation is itself (one
+// double in 2^23 ends in that pattern), v moves up by one unit
+__device__ __forceinline__ split64 split_negatable(long long v) { return split_of(v + ((int)v == INT_MIN ? 1 : 0)); }
 // a b + c, one 32 x 32 + 64-bit multiply-add
 __device__ __forceinline__ long long mad_wide(int a, int b, long long c)
 {
@@ -63,7 +68,9 @@ __device__ __forceinline__ long long add_high(long long hi, long long cross)
 }
 
 // High words of the 128-bit products of z and w, without their low x low terms (below a quarter unit),
-// rounded to nearest; hx, hy: FX_UP or FX_DOWN, the rounding of a tie in each component.
+// rounded to nearest; hx, hy: FX_UP or FX_DOWN, the rounding of a tie in each component.  w's halves
+// are negated in 32 bits: its imaginary part's low half must not be INT_MIN (split_negatable, and
+// split_scaled for the tables).
 //
 // Ties matter: at k = 0 the twiddle is 1 and the product a plain shift, a quarter of whose results are
 // ties.  Always resolved one way they leave a bias of an eighth of a unit in every such product of

@@ -508,7 +508,7 @@ __device__ __forceinline__ int multiply(const FixedArgs &a, const void *gt, int 
         const int xr = mult_fixed(gk.x, m), xi = mult_fixed(gk.y, mi), xm = max(xr, xi);
         m >>= min(xm - xr, 63);
         mi >>= min(xm - xi, 63);
-        const split64 sr = split_of(m), si = split_of(mi);
+        const split64 sr = split_of(m), si = split_negatable(mi);
         r = cmulw(z, make_int4(sr.h, sr.l, si.h, si.l), FX_UP, FX_UP);
         return xm;
     } else {
