@@ -242,9 +242,10 @@ conv_status conv_multi_workspace_size(const conv_plan_t *plans, int count, int b
  *   batch is limited by the array's size, not by the plan's batch_max.
  *   Returns CONV_EINVAL for whatever conv_apply rejects (NULL or aliased pointers, u, out or mask
  *   not aligned to its element size), with a message giving both sizes when the plan and batch
- *   need more than 32 MiB of workspace (conv_workspace_size), and when per-pass timing is enabled
- *   on the plan.  Returns CONV_ECUDA when the array's address could not be looked up at plan
- *   creation.
+ *   need more than 32 MiB of workspace, and when per-pass timing is enabled on the plan.  That need
+ *   is conv_workspace_size, but for FP64 Helmholtz R2C plans whose scratch lines do not fit behind
+ *   the spectra: those run on complex lines without them (the same result to rounding).  Returns
+ *   CONV_ECUDA when the array's address could not be looked up at plan creation.
  *   All calls share the one array: calls that overlap on the GPU (other streams, other threads)
  *   race and corrupt each other's results; serialise them.  The array keeps the last call's
  *   contents; nothing in it needs to start at zero, since each call writes every element it

@@ -51,14 +51,8 @@ extern "C" conv_status conv_apply_noalloc(conv_plan_t p, const void *u, const vo
     if (rc != CONV_OK || batch == 0) return rc;
     // Helmholtz R2C in fixed point: where the split column pass's scratch lines do not fit behind the
     // spectra, the passes on complex lines take the call (the spectra's room holds theirs)
-    const bool split = p->r2c_split;
-    if (p->fixed && workspace_bytes(p, batch) > WSCONV_NOALLOC_SCRATCH_BYTES) p->r2c_split = false;
-    struct Restore {
-        conv_plan_s *p;
-        bool split;
-        ~Restore() { p->r2c_split = split; }
-    } restore{p, split};
-    const size_t need = workspace_bytes(p, batch);
+    const bool split = p->r2c_split && !(p->fixed && workspace_bytes(p, batch) > WSCONV_NOALLOC_SCRATCH_BYTES);
+    const size_t need = workspace_bytes(p, batch, split);
     if (need > WSCONV_NOALLOC_SCRATCH_BYTES)
         return fail(CONV_EINVAL, "conv_apply_noalloc: this plan and batch need " + std::to_string(need) +
                                      " bytes of workspace, above the fixed " +
@@ -69,5 +63,7 @@ extern "C" conv_status conv_apply_noalloc(conv_plan_t p, const void *u, const vo
     if (dev != p->device) return fail(CONV_EINVAL, "the current device is not the plan's device");
     // Every element the column pass reads was written by the row pass of the same call, so the
     // array needs no clearing between calls.
-    return launch_pipeline(p, u, mask, out, batch, 1.0, 0.0, 0.0, ws, reinterpret_cast<cudaStream_t>(stream));
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    if (p->fixed && !p->long_lines) return launch_fixed(p, u, mask, out, batch, 1.0, 0.0, 0.0, split, ws, st);
+    return launch_pipeline(p, u, mask, out, batch, 1.0, 0.0, 0.0, ws, st);
 }

@@ -694,7 +694,7 @@ conv_status launch_pipeline(conv_plan_s *p, const void *u, const void *mask, voi
                             double alpha_re, double alpha_im, double beta, void *ws, cudaStream_t st)
 {
     if (p->long_lines) return long_lines_apply(p, u, mask, out, batch, alpha_re, alpha_im, beta, ws, st);
-    if (p->fixed) return launch_fixed(p, u, mask, out, batch, alpha_re, alpha_im, beta, ws, st);
+    if (p->fixed) return launch_fixed(p, u, mask, out, batch, alpha_re, alpha_im, beta, p->r2c_split, ws, st);
     conv_status rc = CONV_OK;
     if (p->fused)
         WSC_DISPATCH_FUSED(p->prec, p->elems, p->ed, false,

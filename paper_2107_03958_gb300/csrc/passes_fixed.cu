@@ -155,10 +155,10 @@ conv_status set_all_attrs_fixed(int smem)
 }
 
 conv_status launch_fixed(conv_plan_s *p, const void *u, const void *mask, void *out, int batch, double are, double aim,
-                         double beta, void *ws, cudaStream_t st)
+                         double beta, bool split, void *ws, cudaStream_t st)
 {
     conv_status rc = CONV_OK;
-    WSC_FIXED_DISPATCH(fixed_ll(p), rc = run_fixed<LL_>(p, u, mask, out, batch, are, aim, beta, ws, st));
+    WSC_FIXED_DISPATCH(fixed_ll(p), rc = run_fixed<LL_>(p, u, mask, out, batch, are, aim, beta, split, ws, st));
     return rc;
 }
 

@@ -2,6 +2,6 @@
 #include "passes_fixed_launch.cuh"
 
 namespace wsc {
-template conv_status run_fixed<0>(conv_plan_s *, const void *, const void *, void *, int, double, double, double, void *, cudaStream_t);
+template conv_status run_fixed<0>(conv_plan_s *, const void *, const void *, void *, int, double, double, double, bool, void *, cudaStream_t);
 template conv_status set_attrs_fixed<0>(int);
 }  // namespace wsc

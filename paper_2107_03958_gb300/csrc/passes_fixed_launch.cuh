@@ -48,7 +48,7 @@ template <int LL> conv_status set_attrs_fixed(int smem)
 
 template <int LL>
 conv_status run_fixed(conv_plan_s *p, const void *u, const void *mask, void *out, int batch, double are, double aim,
-                      double beta, void *ws, cudaStream_t st)
+                      double beta, bool split, void *ws, cudaStream_t st)
 {
     const int n = p->n, L = p->M, h = p->h;
     const double sc = 1.0 / ((double)L * (double)L);
@@ -90,13 +90,13 @@ conv_status run_fixed(conv_plan_s *p, const void *u, const void *mask, void *out
     a.out = ws;
     a.vec32 = pairs32(ws);
     if (run & 1) {
-        if (r2r || p->r2c_split) launch(mask ? fixed_rows_fwd<LL, FIN_PAIR, true>() : fixed_rows_fwd<LL, FIN_PAIR, false>(), p->rows, 1, batch * ((n + 1) / 2));
+        if (r2r || split) launch(mask ? fixed_rows_fwd<LL, FIN_PAIR, true>() : fixed_rows_fwd<LL, FIN_PAIR, false>(), p->rows, 1, batch * ((n + 1) / 2));
         else if (in_real) launch(mask ? fixed_rows_fwd<LL, FIN_REAL, true>() : fixed_rows_fwd<LL, FIN_REAL, false>(), p->rows, 1, batch * n);
         else launch(mask ? fixed_rows_fwd<LL, FIN_CPLX, true>() : fixed_rows_fwd<LL, FIN_CPLX, false>(), p->rows, 1, batch * n);
     }
     if (ev) cudaEventRecord(ev[1], st);
     a.in = p->w_in ? p->w_in : ws;
-    if (p->r2c_split) {
+    if (split) {
         // W2 follows W on the next even element, the scratch lines after the batch's 3 h n + 1 values
         double2 *w = reinterpret_cast<double2 *>(ws);
         a.out = w + (((size_t)batch * h * n + 1) & ~(size_t)1);
@@ -111,9 +111,9 @@ conv_status run_fixed(conv_plan_s *p, const void *u, const void *mask, void *out
     if (run & 4) {
         a.in = a.out;
         a.out = out;
-        a.vec32 = p->r2c_split ? reinterpret_cast<uintptr_t>(a.in) % 32 == 0 : pairs32(a.in);
+        a.vec32 = split ? reinterpret_cast<uintptr_t>(a.in) % 32 == 0 : pairs32(a.in);
         if (r2r) launch(beta != 0.0 ? fixed_rows_inv<LL, FOUT_R2R, true>() : fixed_rows_inv<LL, FOUT_R2R, false>(), p->inv, 1, batch * ((n + 1) / 2));
-        else if (p->r2c_split) launch(beta != 0.0 ? fixed_rows_inv<LL, FOUT_SPLIT, true>() : fixed_rows_inv<LL, FOUT_SPLIT, false>(), p->inv, 1, batch * n);
+        else if (split) launch(beta != 0.0 ? fixed_rows_inv<LL, FOUT_SPLIT, true>() : fixed_rows_inv<LL, FOUT_SPLIT, false>(), p->inv, 1, batch * n);
         else if (in_real) launch(beta != 0.0 ? fixed_rows_inv<LL, FOUT_REAL, true>() : fixed_rows_inv<LL, FOUT_REAL, false>(), p->inv, 1, batch * n);
         else launch(beta != 0.0 ? fixed_rows_inv<LL, FOUT_CPLX, true>() : fixed_rows_inv<LL, FOUT_CPLX, false>(), p->inv, 1, batch * n);
     }

@@ -68,7 +68,7 @@ size_t spectrum_elems(const conv_plan_s *p)
     return (size_t)(p->io == CONV_IO_R2R ? p->h : p->M) * p->n;
 }
 
-size_t workspace_bytes(const conv_plan_s *p, int batch)
+size_t workspace_bytes(const conv_plan_s *p, int batch, bool split)
 {
     if (p->long_lines) return batch > 0 ? long_lines_ws_bytes(p) : 0;  // densities run one at a time
     const size_t esz = p->prec == CONV_P_FP64 ? 16 : 8;
@@ -76,7 +76,7 @@ size_t workspace_bytes(const conv_plan_s *p, int batch)
     // use no more of them than columns, rounded up to whole CTAs
     size_t lines = p->split_scratch_elems;
     if (p->fixed) lines = std::min(lines, ((size_t)batch * p->h + p->cols.groups) * p->M);
-    const size_t scratch = p->r2c_split && lines ? lines + 1 : 0;
+    const size_t scratch = split && lines ? lines + 1 : 0;
     return batch > 0 ? (spectrum_elems(p) * (size_t)batch + scratch) * esz : 0;
 }
 

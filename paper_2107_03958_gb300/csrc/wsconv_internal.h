@@ -228,8 +228,9 @@ conv_status select_transform(conv_plan_s *p);
 // passes_fixed.cu
 bool fixed_configure(conv_plan_s *p, int smem_optin, int sms);
 conv_status set_all_attrs_fixed(int smem);
+// split: the split R2C passes (p->r2c_split), or false: the same plan's passes on complex lines
 conv_status launch_fixed(conv_plan_s *p, const void *u, const void *mask, void *out, int batch, double are,
-                         double aim, double beta, void *ws, cudaStream_t st);
+                         double aim, double beta, bool split, void *ws, cudaStream_t st);
 void fixed_twiddles(const FixedDesc &d, std::vector<int> &tab);
 // exp(-2 pi i t / L) = (re[t], im[t]), t < L.  conv(x) turns a long double cosine or sine into T and is called,
 // like the two functions, on the first octant (quadrant, half) alone; the rest are its values with
@@ -279,7 +280,11 @@ void long_lines_destroy(conv_plan_s *p);
 size_t long_lines_ws_bytes(const conv_plan_s *p);
 conv_status long_lines_apply(conv_plan_s *p, const void *u, const void *mask, void *out, int batch, double are,
                              double aim, double beta, void *ws, cudaStream_t st);
-size_t workspace_bytes(const conv_plan_s *p, int batch);  // plan.cu: conv_workspace_size
+size_t workspace_bytes(const conv_plan_s *p, int batch, bool split);  // split: as launch_fixed's
+inline size_t workspace_bytes(const conv_plan_s *p, int batch)  // plan.cu: conv_workspace_size
+{
+    return workspace_bytes(p, batch, p->r2c_split);
+}
 bool fault_take(int kind);                      // plan.cu: consume one armed injected fault
 // plan.cu: free a plan; wait_device = false only when no queued or running work uses it
 void plan_release(conv_plan_s *p, bool wait_device);
