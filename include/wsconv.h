@@ -298,11 +298,14 @@ typedef struct {
     int nstages;
     int radices[16];
     size_t ghat_bytes, workspace_bytes;
+    /* threads per line, and lines per CTA: the most a CTA holds, of which small grids use fewer to
+     * reach every SM */
     int threads_rows, groups_rows, threads_cols, groups_cols;
     int transform_len;   /* points per line in the passes: M = n b, or 2n when compact */
     int compact;         /* CONV_PLAN_COMPACT was set */
     int elems;           /* complex elements per thread in the transform kernels (0: generic) */
-    int smem_twiddles;   /* twiddle table staged in shared memory */
+    int smem_twiddles;   /* twiddle table staged in shared memory (FP64 lines of static_len points:
+                          * the part that the radix-16 stages read most) */
     int fused;           /* fused passes (global-memory first/last stages) */
     int static_log2;     /* log2 of the transform length when it is a power of two whose stage
                           * structure is fixed at compile time (fused passes), else 0 */

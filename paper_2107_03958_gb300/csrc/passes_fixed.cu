@@ -135,7 +135,7 @@ bool fixed_configure(conv_plan_s *p, int smem_optin, int sms)
     p->sms = sms;
     p->fixed = p->fused = true;
     p->elems = 16;
-    p->tws = false;
+    p->tws = ll != 0;  // the radix-16 stages' (fixed_tw_smem)
     int l2 = 0;
     while ((1 << l2) < L) ++l2;
     p->ed = ll ? 1000 + l2 : 0;
