@@ -75,7 +75,16 @@ __device__ __forceinline__ typename cvec<T>::t *setup_smem(const PassArgs<T> &a,
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V *base = reinterpret_cast<V *>(smem_raw);
     if (TWS) {
-        for (int t = threadIdx.x; t < a.tw_len; t += blockDim.x) base[t] = __ldg(&a.tw[t]);
+        // eight loads in flight a thread: a CTA of one short line has few threads, and copying the table
+        // entry by entry it waited on L2 for each round
+        for (int t = threadIdx.x; t < a.tw_len; t += 8 * blockDim.x) {
+            V r[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) r[i] = __ldg(&a.tw[min(t + i * (int)blockDim.x, a.tw_len - 1)]);
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (t + i * (int)blockDim.x < a.tw_len) base[t + i * blockDim.x] = r[i];
+        }
         __syncthreads();
         twp = base;
         base += a.tw_len;

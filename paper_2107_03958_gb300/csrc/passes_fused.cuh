@@ -747,7 +747,11 @@ conv_status run_fused(conv_plan_s *p, const void *u, const void *mask, void *out
     // Groups per CTA: as many as the shape holds, unless fewer than half the SMs would then get a CTA:
     // one small density's rows run faster spread over the chip (C2C batch 1, passes 1 / 2 / 3:
     // n = 512, 64 CTAs of 8 groups -> 128 of 4, 16.4 / 12.5 / 12.3 -> 12.8 / 10.8 / 10.2 us; n = 256 13.7 / 8.3 / 10.2 ->
-    // 12.2 / 8.8 / 8.2 us), while at 128 CTAs of 8 groups (batch 8 of n = 256) 147 of 7 gain nothing
+    // 12.2 / 8.8 / 8.2 us), while at 128 CTAs of 8 groups (batch 8 of n = 256) 147 of 7 gain nothing.  A CTA
+    // keeps at least a warp of threads: lines of 72 to 288 points have 3 to 12, and spread one to a CTA they
+    // made an isolated call slower than eight to a CTA (device time of a C2C call at n = 24 / 48 / 96: 43 /
+    // 46 / 50 us with eight, 47 / 54 / 57 with one, 43 / 51 / 53 with a warp's worth and the table copied in
+    // batches; among others 27 / 31 / 34, 24 / 30 / 30 and 23 / 30 / 31)
     struct Geo {
         unsigned grid, threads;
         size_t smem;
@@ -756,7 +760,7 @@ conv_status run_fused(conv_plan_s *p, const void *u, const void *mask, void *out
     const bool may_early = may_launch_early(st);
     auto geo = [&](const LaunchShape &S, int units) {
         const bool few = (units + S.groups - 1) / S.groups < p->sms / 2;
-        const int G = few ? (units + p->sms - 1) / p->sms : S.groups;
+        const int G = few ? std::min(S.groups, std::max((units + p->sms - 1) / p->sms, (32 + S.tpt - 1) / S.tpt)) : S.groups;
         const long long need = (units + G - 1) / G, most = (long long)S.max_ctas * (S.groups / G);
         return Geo{(unsigned)std::min(need, most), (unsigned)(S.tpt * G), S.smem - S.smem_group * (S.groups - G), may_early && need <= p->sms};
     };
