@@ -409,8 +409,8 @@ static bool configure(conv_plan_s *p, const Candidate &c, int smem_optin, int sm
     const int M = p->M, n = p->n;
     p->fixed = false;
     // FP64 lines of 32 to 8192 points (as far as two buffers fit beside each other, for the lengths
-    // without kernels of their own) run in fixed point: 3.6 to 4.7 times the FP64 stages' rate from n = 256 on,
-    // 1.6 times at n = 64 (n = 4096, batch 16: 125.3 -> 27.6 ms; n = 480, period 3, batch 8: 2266 -> 592 us)
+    // without kernels of their own) run in fixed point: 3.7 to 5.8 times the FP64 stages' rate from n = 256 on,
+    // 1.6 times at n = 64 (n = 4096, batch 16: 125.2 -> 27.1 ms; n = 480, period 3, batch 8: 2263 -> 606 us)
     p->multi_ok = true;
     if (p->prec == CONV_P_FP64 && E == 16) {
         p->multi_ok = multi_length64(p, smem_optin);
@@ -591,6 +591,8 @@ static conv_status device_limits(conv_plan_s *p, int &smem_optin, int &sms)
 // of each pass.  Environment overrides for experiments: WSCONV_ELEMS, WSCONV_FUSED (0/1),
 // WSCONV_TWS (0: no pass keeps its table in shared memory), WSCONV_PF (0/1: prefetch in no / every
 // pass), WSCONV_GROUPS (1: one transform per CTA), WSCONV_CFG ("r,c,i": the CFG_* bits per pass).
+// The last four have no effect on the fixed-point passes, whose shapes follow from the length; an
+// FP64 plan takes other passes with WSCONV_ELEMS = 12, 24, 8 or 0, or WSCONV_FUSED = 0 or 2.
 // Lines that one CTA cannot hold (or, with WSCONV_LONG_LINES=1, any line: tests) take the
 // four-step FP64 line pipeline of fsmask.cu (p->long_lines).
 static bool factor_235(int L)

@@ -51,10 +51,11 @@ template <typename T, int ED> __host__ __device__ constexpr bool pingpong_ok() {
 // set-up (shared memory, twiddle copies, which only read the plan's tables) overlap the tail of its
 // predecessor on the stream.  Every pass kernel calls pdl_wait() before it touches anything its
 // predecessors wrote or read, on every path; what follows it on the stream then also follows them.
-// Used where a launch's CTAs all run at once (the passes of a small grid are a few microseconds each:
-// FP32 n = 64 29.9 -> 22.2 us, FP64 n = 64 31.0 -> 27.1, FP64 n = 256 batch 16 90.8 -> 84.8) and not under
-// capture (the FP64 LS step graphs at n = 512: 2.69 -> 2.81 ms a solve) or for grids of several rounds,
-// where waiting CTAs gain nothing.
+// Used where a launch's CTAs all run at once (the passes of a small grid are a few microseconds each;
+// calls in a row, plain -> early: FP32 n = 64 26.7 -> 21.6 us, FP64 n = 64 34 -> 31, FP64 n = 256 batch 16 89 -> 85;
+// an isolated call gains up to 6 us at the compile-time lengths, C2C FP32 n = 128 34 -> 28, and loses up to
+// 5 on FP32 runtime stages, C2C n = 48 46 -> 51) and not under capture (the FP64 LS step graphs at n = 512:
+// 2.69 -> 2.81 ms a solve) or for grids of several rounds, where waiting CTAs gain nothing.
 template <class... P, class... A>
 inline cudaError_t launch_pass(void (*kernel)(P...), bool early, unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args)
 {
@@ -119,7 +120,7 @@ bool encode_rows_map(CUtensorMap *m, const void *base, unsigned long long words,
 
 // Stage structure of one fixed-point transform (kernel parameter).  The first stage has no
 // twiddles; the powers of two come first (16s, then the rest), so only radix-3 and radix-5 stages
-// see an Ns that is not a power of two.  Twiddle table: for stage s >= 1, tw_variants(R) copies of
+// see an Ns that is not a power of two.  Twiddle table: for stage s >= 1, fixed_variants(R) copies of
 // [w^k | w^2k | ... | w^(R-1)k], k < Ns, w = exp(-2 pi i / (Ns R)), copy v scaled by 2^(62 - v): the
 // product's high word is then the product over 2^(2 + v).
 struct FixedDesc {
@@ -193,7 +194,8 @@ struct conv_plan_s {
     // FP32 copy for FP32 plans (float or float2)
     void *ghat32 = nullptr;
     size_t ghat_bytes = 0;
-    // twiddle table exp(-2 pi i t / M), t in [0, M), plan precision
+    // per-stage twiddle blocks: FFTDesc's in the plan's precision, or FixedDesc's as (re h, re l, im h,
+    // im l) 32-bit halves (fixed)
     void *tw = nullptr;
     void *ws = nullptr;
     size_t ws_bytes = 0;
